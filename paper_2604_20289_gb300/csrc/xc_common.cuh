@@ -181,7 +181,7 @@ __device__ __forceinline__ int4 token_pos(const EpiParams &p, int row) {
 enum { EPI_BIAS = XC_EPI_BIAS, EPI_GELU = XC_EPI_GELU, EPI_RESID_GATE = XC_EPI_RESID_GATE,
        EPI_RESID_CACHE = XC_EPI_RESID_CACHE, EPI_QKV_ROPE = 16 };
 
-// Runs of W = 8 or 16 consecutive elements (16-byte aligned).
+// Runs of W = 8 or 16 (float: also 4) consecutive elements (16-byte aligned).
 template <typename T, int W>
 __device__ __forceinline__ void loadW(const T *p, float (&v)[W]) {
     if constexpr (W == 16) {
@@ -195,6 +195,9 @@ __device__ __forceinline__ void loadW(const T *p, float (&v)[W]) {
             v[2 * j] = f.x;
             v[2 * j + 1] = f.y;
         }
+    } else if constexpr (W == 4) {
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     } else {
         const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
@@ -213,6 +216,8 @@ __device__ __forceinline__ void storeW(T *p, const float (&v)[W]) {
             w[j] = *reinterpret_cast<uint32_t *>(&h);
         }
         *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else if constexpr (W == 4) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
     } else {
         reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
         reinterpret_cast<float4 *>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
@@ -220,7 +225,7 @@ __device__ __forceinline__ void storeW(T *p, const float (&v)[W]) {
 }
 
 // Fused GEMM epilogue on one run of W consecutive output columns
-// [col, col + W) of one row (W = 8 or 16, col a multiple of W).
+// [col, col + W) of one row (W = 4 (float), 8 or 16, col a multiple of W).
 template <int EPI, typename T, int W>
 __device__ __forceinline__ void epilogue_run(const EpiParams &p, int row, int col, float (&acc)[W]) {
     if (row >= p.M) return;
@@ -281,9 +286,4 @@ __device__ __forceinline__ void epilogue_run(const EpiParams &p, int row, int co
         storeW<T, W>(dst + (size_t)row * d + c, acc);
     }
 }
-template <int EPI, typename T>
-__device__ __forceinline__ void epilogue16(const EpiParams &p, int row, int col, float (&acc)[16]) {
-    epilogue_run<EPI, T, 16>(p, row, col, acc);
-}
-
 }  // namespace xc
