@@ -430,20 +430,7 @@ void gate_bind_scratch(GateArgs &g, const GateGeom &gg, void *scratch) {
 template <typename T>
 static cudaError_t cluster_launch(void (*kern)(GateArgs), const GateArgs &g, cudaStream_t st) {
     if (g.R < 1 || g.R > GATE_MAX_CLUSTER) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.V * g.n_slices * g.R);
-    cfg.blockDim = dim3(GATE_THREADS);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)g.R;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, g);
+    return launch_pdl_cluster(kern, (unsigned)g.R, dim3(g.V * g.n_slices * g.R), dim3(GATE_THREADS), 0, st, g);
 }
 template <typename T>
 cudaError_t gate_launch(const GateArgs &g, cudaStream_t st) {

@@ -2,69 +2,91 @@
 //
 //   C[M][N] = epilogue(A[M][K] @ Wt[N][K]^T), fp32 accumulation in TMEM.
 //
-// Persistent: one CTA per SM walks the 128 x BN output tiles round-robin
-// (n fastest, so the CTAs running at the same time share A tiles in L2).
-// Warp roles (320 threads):
-//   warp 0, lane 0 : TMA producer, STAGES-deep ring of (A 128x64, B BNx64)
+// Tilings, picked by gemm_tc_bn:
+//   pair   (BN = 256) a cluster of two CTAs works on one 256 x 256 tile with
+//          tcgen05.mma.cta_group::2: each CTA loads its 128 rows of A and
+//          half of B's 256 rows, 32 KB per 64-deep k step where a CTA of its
+//          own with a 128 x 256 tile loads 48 KB -- the operand feed from L2
+//          bounds the main loop, so a third fewer bytes per MMA is what the
+//          pair is for (and six ring stages fit instead of four);
+//   single (BN = 128, 64) one CTA per 128 x BN tile, for GEMMs with too few
+//          256 x 256 tiles to fill the pairs.  With few tiles a k step waits
+//          for the latency of its loads (some 2200 cycles over the ring's
+//          depth): 64-wide tiles put twice the CTAs and eight stages to work.
+// Persistent: the CTAs (pairs) walk the output tiles in grouped super-rows
+// (tile_at).  Warp roles (320 threads per CTA):
+//   warp 0         : TMA producer, STAGES-deep ring of (A 128x64, B 128x64)
 //                    tiles in 128B-swizzled shared memory, continuous across
-//                    output tiles;
-//   warp 1         : allocates TMEM (two BN-column accumulators) and issues
-//                    tcgen05.mma (M=128, N=BN, K=16; 4 per 64-wide k-tile)
-//                    into the free accumulator from a converged warp;
+//                    output tiles; in a pair both CTAs' bytes are counted on
+//                    the leader's full barriers;
+//   warp 1         : allocates TMEM (two accumulators) and issues
+//                    tcgen05.mma (K=16; 4 per 64-wide k-tile) into the free
+//                    accumulator from a converged warp; in a pair the
+//                    leader's alone, its commits arriving in both CTAs;
 //   warps 2..9     : epilogue, two warps per TMEM lane quadrant, half of the
 //                    columns each, in 32 x 32 blocks: thread = row, the
 //                    block's residual operands arrive in shared memory by
 //                    TMA, the fused epilogue (bias / GELU / gated residual /
 //                    residual cache / RoPE) runs in registers, and the bf16
 //                    block leaves by a TMA store from a 64B-swizzled staging
-//                    buffer.  The accumulator is released after its last
-//                    TMEM read, so the epilogue of tile i overlaps the main
-//                    loop of tile i + 1.
+//                    buffer.  The accumulator is released (to the leader)
+//                    after its last TMEM read, so the epilogue of tile i
+//                    overlaps the main loop of tile i + 1.
 // The skip flag of the block lets the whole recompute path early-exit when
 // the gate chose reuse (Eq. 4), so decisions never return to the host.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <unordered_map>
 
+#include "xc_kernels.cuh"
 #include "xc_ptx.cuh"
 
 namespace xc {
 
 constexpr int GEMM_BM = 128;
 constexpr int GEMM_BK = 64;
+constexpr int GEMM_THREADS = 320;              // producer warp, MMA warp, 8 epilogue warps
 constexpr int GEMM_SMEM_LIMIT = 232448;        // dynamic shared memory per CTA on this part
 constexpr int EPI_BLOCK_BYTES = 32 * 32 * 2;   // one 32 x 32 bf16 block
 
-// Residual-cache epilogue with 256-wide tiles: the residual and block-input
-// blocks are loaded into the two buffers that then stage the output and
-// r_hat, so the main loop keeps four pipeline stages in shared memory (the
-// next blocks' loads wait until the stores have read the buffers).
-template <int EPI, int BN>
-__host__ __device__ constexpr bool epi_shared() {
-    return EPI == EPI_RESID_CACHE && BN == 256;
-}
-// Staging blocks per epilogue warp: residual cache: out, r_hat, resid, x_in
-// (2 when shared); gated residual: out, resid; the others: out,
-// double-buffered.
-template <int EPI, int BN>
-__host__ __device__ constexpr int epi_blocks() {
-    return (EPI == EPI_RESID_CACHE && !epi_shared<EPI, BN>()) ? 4 : 2;
-}
+// Staging ring of an epilogue warp: SLOTS slots of one 32 x 32 block (residual
+// cache: two, out / r_hat), used in block order across output tiles.  The
+// residual operands of a block land in its slot AHEAD blocks before they are
+// needed, the output replaces them in place (a lane touches its own row
+// only), and a slot is loaded or written again once its store has been read.
+template <int BN, int EPI, bool DEEP>
+struct EpiRing {
+    static constexpr bool RES = EPI == EPI_RESID_GATE || EPI == EPI_RESID_CACHE;
+    static constexpr bool CACHE = EPI == EPI_RESID_CACHE;
+    // Two slots leave the main loop six ring stages, four (DEEP) five; a gated
+    // residual with a short K gains more from loading two blocks ahead.  Two /
+    // four slots measured: 8064 x 1536 x 512 13.3 / 14.4 us, 12960 x 8960 x
+    // 1536 + GELU 187 / 190; gated 6000 x 4096 x 512 28.0 / 25.9, gated 4000
+    // x 256 x 6976 23.9 / 26.6
+    static constexpr int SLOTS = DEEP ? 4 : 2;
+    static constexpr int AHEAD = SLOTS / 2;
+    static constexpr int SLOT_BYTES = (CACHE ? 2 : 1) * EPI_BLOCK_BYTES;
+};
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool DEEP>
 struct GemmTile {
+    static constexpr bool PAIR = BN == 256;            // two CTAs per tile
+    static constexpr int BM = PAIR ? 2 * GEMM_BM : GEMM_BM;
     static constexpr int A_BYTES = GEMM_BM * GEMM_BK * 2;
-    static constexpr int B_BYTES = BN * GEMM_BK * 2;
+    static constexpr int B_BYTES = (PAIR ? 128 : BN) * GEMM_BK * 2;   // pair: this CTA's half of B's rows
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int EPI_BYTES = 8 * epi_blocks<EPI, BN>() * EPI_BLOCK_BYTES;
-    static constexpr int BAR_BYTES = 512;
-    static constexpr int FIT = (GEMM_SMEM_LIMIT - 1024 - BAR_BYTES - EPI_BYTES) / STAGE_BYTES;
-    static constexpr int STAGES = FIT > 6 ? 6 : FIT;
+    static constexpr int EPI_BYTES = 8 * EpiRing<BN, EPI, DEEP>::SLOTS * EpiRing<BN, EPI, DEEP>::SLOT_BYTES;
+    static constexpr int VEC_BYTES = 8 * 64 * 4;       // bias and gate of a warp's block
+    static constexpr int BAR_BYTES = VEC_BYTES + 512;
+    static constexpr int FIT = (GEMM_SMEM_LIMIT - BAR_BYTES - EPI_BYTES) / STAGE_BYTES;
+    static constexpr int STAGES = FIT > 8 ? 8 : FIT;
     static constexpr int OFF_EPI = STAGES * STAGE_BYTES;                // 1024-aligned
-    static constexpr int BAR_OFFSET = OFF_EPI + EPI_BYTES;
-    static constexpr int SMEM_BYTES = BAR_OFFSET + BAR_BYTES + 1024;   // + alignment slack
+    static constexpr int OFF_VEC = OFF_EPI + EPI_BYTES;
+    static constexpr int BAR_OFFSET = OFF_VEC + VEC_BYTES;
+    static constexpr int SMEM_BYTES = OFF_VEC + BAR_BYTES;
     static constexpr int TMEM_COLS = 2 * BN;                             // double-buffered accumulator
-    static constexpr int EPI_THREADS = 256;
+    static constexpr int EPI_WARPS = PAIR ? 16 : 8;    // that release an accumulator
     static_assert(STAGES >= 3, "main-loop ring too shallow");
     static_assert(SMEM_BYTES <= GEMM_SMEM_LIMIT, "shared memory");
 };
@@ -75,11 +97,6 @@ struct EpiMaps {
     CUtensorMap out[3];
     CUtensorMap rhat, resid, xin;
 };
-
-__device__ __forceinline__ uint8_t *align1024(uint8_t *p) {
-    const uint32_t s = smem_u32(p);
-    return p + ((1024u - (s & 1023u)) & 1023u);
-}
 
 // Byte offset of 16-byte chunk k (0..3) of row r in a 64B-swizzled 32 x 32
 // bf16 block (the layout TMA reads and writes with CU_TENSOR_MAP_SWIZZLE_64B).
@@ -96,6 +113,32 @@ __device__ __forceinline__ void bulk_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// (a, b) += (x, y), (a, b) = (x a + r, y b + s): packed fp32 pairs
+__device__ __forceinline__ void add2(float &a, float &b, float x, float y) {
+    const float2 t = __fadd2_rn(make_float2(a, b), make_float2(x, y));
+    a = t.x;
+    b = t.y;
+}
+__device__ __forceinline__ void fma2(float &a, float &b, float x, float y, float r, float s) {
+    const float2 t = __ffma2_rn(make_float2(x, y), make_float2(a, b), make_float2(r, s));
+    a = t.x;
+    b = t.y;
+}
+// gelu_tanh_approx of two values (the same operations, packed)
+__device__ __forceinline__ void gelu_tanh_approx2(float &a, float &b) {
+    const float k0 = 0.7978845608028654f;
+    const float2 x = make_float2(a, b);
+    const float2 c = __fmul2_rn(make_float2(0.044715f, 0.044715f), x), x2 = __fmul2_rn(x, x);
+    const float2 u = __fmul2_rn(make_float2(k0, k0), __ffma2_rn(c, x2, x));
+    float2 t;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t.x) : "f"(u.x));
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t.y) : "f"(u.y));
+    const float2 hx = __fmul2_rn(make_float2(0.5f, 0.5f), x);
+    const float2 y = __ffma2_rn(hx, t, hx);
+    a = y.x;
+    b = y.y;
+}
 
 // 32 bf16 of row r from a swizzled block -> float
 __device__ __forceinline__ void read_row32(const uint8_t *blk, int r, float (&v)[32]) {
@@ -126,45 +169,75 @@ __device__ __forceinline__ void write_row32(uint8_t *blk, int r, const float (&v
 }
 
 // Persistent tile order: tile t -> (m block, n block).  Tiles go in
-// super-rows of GEMM_GROUP_M m blocks with m varying fastest inside a
-// super-row, so the tiles in flight at one time (one per SM) share
-// GEMM_GROUP_M row blocks of A and a few column blocks of B -- an
+// super-rows of 16 x 128 rows with m varying fastest inside a
+// super-row, so the tiles in flight at one time (one per SM or pair) share
+// the super-row's row blocks of A and a few column blocks of B -- an
 // L2-resident working set -- instead of all of B streaming through L2 for
 // every row of m blocks (row-major order re-read B from DRAM once per 2-3
 // m-block rows on the large-N projections).
-constexpr int GEMM_GROUP_M = 16;
-__device__ __forceinline__ void tile_mn(int tile, int tiles_m, int tiles_n, int &mb, int &nb) {
-    const int per = GEMM_GROUP_M * tiles_n;
-    const int grp = tile / per;
-    const int first = grp * GEMM_GROUP_M;
-    const int gm = min(GEMM_GROUP_M, tiles_m - first);
-    const int loc = tile - grp * per;
-    mb = first + loc % gm;
-    nb = loc / gm;
+// Pairs: tiles from n_full on (the remainder of the last round, when it would
+// leave more than half of the pairs idle) are cut into two 256 x 128 halves,
+// items n_full, n_full + 1, ... of the walk: such a round loads 24 KB instead
+// of 32 per k step and costs about 0.6 of a full one.
+struct TileWalk {
+    int tiles_m, tiles_n, n_full, n_items;
+};
+struct Tile {
+    int m0, n0, w;                                   // first row, first column, columns
+};
+template <int BM, int BN>
+__device__ __forceinline__ Tile tile_at(const TileWalk &tw, int item) {
+    constexpr int GROUP_M = 16 * GEMM_BM / BM;
+    Tile r{0, 0, BN};
+    int t = item, sub = 0;
+    if (BN == 256 && item >= tw.n_full) {
+        t = tw.n_full + ((item - tw.n_full) >> 1);
+        sub = (item - tw.n_full) & 1;
+        r.w = 128;
+    }
+    const int per = GROUP_M * tw.tiles_n;
+    const int grp = t / per;
+    const int first = grp * GROUP_M;
+    const int gm = min(GROUP_M, tw.tiles_m - first);
+    const int loc = t - grp * per;
+    r.m0 = (first + loc % gm) * BM;
+    r.n0 = (loc / gm) * BN + sub * 128;
+    return r;
 }
 
-template <int BN, int EPI>
-__global__ void __launch_bounds__(320, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ EpiMaps em, const EpiParams ep, const int K,
+template <int BN, int EPI, bool DEEP>
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
+    gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ WeightMaps tmB,
+                   const __grid_constant__ EpiMaps em, const EpiParams ep, const int K, const TileWalk tw,
                    const uint8_t *__restrict__ skip_flag, int *err) {
+    using G = GemmTile<BN, EPI, DEEP>;
+    if (threadIdx.x == 0) {                           // kernel parameters: nothing a predecessor writes
+        prefetch_tmap(&tmA);
+        prefetch_tmap(BN == 64 ? &tmB.box64 : &tmB.box128);
+    }
     pdl_wait();
-    using G = GemmTile<BN, EPI>;
     if (skip_flag != nullptr && *skip_flag == XC_DEC_SKIP) return;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = align1024(smem_raw);
+    // 1024-byte aligned (128B swizzle atoms): the declared alignment holds for
+    // the window's base; nothing runs if it did not
+    extern __shared__ __align__(1024) uint8_t smem[];
+    if ((smem_u32(smem) & 1023u) != 0) {
+        if (threadIdx.x == 0) atomicOr(err, ERR_BAD_LAUNCH);
+        return;
+    }
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + G::BAR_OFFSET);
     uint64_t *empty = full + G::STAGES;
     uint64_t *acc_full = empty + G::STAGES;    // [2]
     uint64_t *acc_empty = acc_full + 2;        // [2]
-    uint64_t *ld_bar = acc_empty + 2;          // [8] residual operands of an epilogue warp landed
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ld_bar + 8);
+    uint64_t *ld_bar = acc_empty + 2;          // [8][SLOTS] residual operands of an epilogue warp's slot landed
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ld_bar + 8 * EpiRing<BN, EPI, DEEP>::SLOTS);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KT = K / GEMM_BK;
-    const int tiles_n = ep.N / BN;
-    const int tiles_m = (ep.M + GEMM_BM - 1) / GEMM_BM;
-    const int n_tiles = tiles_m * tiles_n;
+    constexpr bool PAIR = G::PAIR;
+    // worker = CTA or CTA pair; rank 0 of a pair leads (issues its MMAs)
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0;
+    const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x, n_workers = PAIR ? gridDim.x >> 1 : gridDim.x;
+    const int row_off = PAIR ? (int)rank * GEMM_BM : 0;      // this CTA's rows of the tile
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < G::STAGES; ++s) {
@@ -173,48 +246,64 @@ __global__ void __launch_bounds__(320, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], G::EPI_THREADS);
+            mbar_init(&acc_empty[b], G::EPI_WARPS);
         }
-        for (int w = 0; w < 8; ++w) mbar_init(&ld_bar[w], 1);
+        for (int w = 0; w < 8 * EpiRing<BN, EPI, DEEP>::SLOTS; ++w) mbar_init(&ld_bar[w], 1);
         mbar_fence_init();
     }
-    if (warp == 1) tmem_alloc(tmem_slot, G::TMEM_COLS);
+    if (warp == 1) {
+        if constexpr (PAIR) tmem_alloc_pair(tmem_slot, G::TMEM_COLS);
+        else tmem_alloc(tmem_slot, G::TMEM_COLS);
+    }
     tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();           // the peer's barriers are initialised too
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int it = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x) {
-                int mb, nb;
-                tile_mn(tile, tiles_m, tiles_n, mb, nb);
-                const int m0 = mb * GEMM_BM, n0 = nb * BN;
-                for (int kt = 0; kt < KT; ++kt, ++it) {
-                    const int s = it % G::STAGES;
-                    const uint32_t ph = (it / G::STAGES) & 1;
-                    if (!mbar_wait(&empty[s], ph ^ 1, err, ERR_WAIT_PRODUCER)) {
-                        ok = false;
-                        break;
-                    }
-                    uint8_t *sa = smem + s * G::STAGE_BYTES;
-                    mbar_expect_tx(&full[s], G::STAGE_BYTES);
-                    tma_load_2d(sa, &tmA, &full[s], kt * GEMM_BK, m0);
-                    tma_load_2d(sa + G::A_BYTES, &tmB, &full[s], kt * GEMM_BK, n0);
+        // The whole warp runs the loop (converged), one elected lane issues.
+        int it = 0;
+        bool ok = true;
+        for (int item = worker; ok && item < tw.n_items; item += n_workers) {
+            const Tile t = tile_at<G::BM, BN>(tw, item);
+            const int m0 = t.m0 + row_off, n0 = PAIR ? t.n0 + (int)rank * (t.w / 2) : t.n0;
+            const int b_rows = PAIR ? t.w / 2 : BN;           // of B
+            const CUtensorMap *tb = b_rows == 128 ? &tmB.box128 : &tmB.box64;
+            const uint32_t bytes = (uint32_t)G::A_BYTES + (uint32_t)b_rows * (GEMM_BK * 2);
+            for (int kt = 0; kt < KT; ++kt, ++it) {
+                const int s = it % G::STAGES;
+                const bool r = mbar_wait(&empty[s], ((it / G::STAGES) & 1) ^ 1, err, ERR_WAIT_PRODUCER);
+                if (!__all_sync(0xffffffffu, r)) {
+                    ok = false;
+                    break;
                 }
+                uint8_t *sa = smem + s * G::STAGE_BYTES;
+                if constexpr (PAIR)
+                    tma_stage_pair_warp(&full[s], map_to_cta(&full[s], 0), rank == 0, 2 * bytes, sa, &tmA, m0,
+                                        sa + G::A_BYTES, tb, n0, kt * GEMM_BK);
+                else
+                    tma_stage_warp(&full[s], bytes, sa, &tmA, m0, sa + G::A_BYTES, tb, n0, kt * GEMM_BK);
             }
-            // Drain: every copy this thread started has landed before exit.
+        }
+        // Drain: every copy this warp started has landed before exit.  A
+        // pair's leader waits for both CTAs' bytes, and the peer leaves only
+        // after it (the cluster barrier at the end); the peer sees no barrier
+        // of its own, so when one of its waits ran out it gives its last
+        // copies a fixed 10 ms.
+        if (rank == 0) {
             for (int j = it - G::STAGES < 0 ? 0 : it - G::STAGES; j < it; ++j)
                 mbar_wait(&full[j % G::STAGES], (j / G::STAGES) & 1, err, ERR_WAIT_PRODUCER);
+        } else if (!ok) {
+            const unsigned long long t0 = global_ns();
+            for (unsigned i = 0; i < WAIT_MAX_ITERS && global_ns() - t0 < 10000000ull; ++i) {
+            }
         }
     } else if (warp == 1) {
         // MMA issue: the whole warp runs the loop (converged) and one elected
         // lane issues each tcgen05 instruction, so issue keeps pace while the
         // epilogue warps of the same sub-partitions are busy.
-        {
-            constexpr uint32_t idesc = idesc_bf16(GEMM_BM, BN, false, false);
+        if (rank == 0) {
             auto wait = [&](uint64_t *b, uint32_t parity) {
                 const bool r = mbar_wait(b, parity, err, ERR_WAIT_MMA);
                 return __all_sync(0xffffffffu, r);
@@ -223,9 +312,11 @@ __global__ void __launch_bounds__(320, 1)
             const uint64_t d0 = sdesc_sw128(smem_u32(smem), 16, 1024);
             int it = 0, local = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++local) {
+            for (int item = worker; ok && item < tw.n_items; item += n_workers, ++local) {
                 const int buf = local & 1;
                 const uint32_t use = (uint32_t)(local >> 1);
+                const uint32_t idesc = BN == 256 && item >= tw.n_full ? idesc_bf16(G::BM, 128, false, false)
+                                                                      : idesc_bf16(G::BM, BN, false, false);
                 if (!wait(&acc_empty[buf], (use & 1) ^ 1)) break;
                 tc_fence_after();
                 const uint32_t acc = tmem + buf * BN;
@@ -239,56 +330,58 @@ __global__ void __launch_bounds__(320, 1)
                     const uint64_t da = d0 + (uint64_t)((s * G::STAGE_BYTES) >> 4);
                     const uint64_t db = da + (uint64_t)(G::A_BYTES >> 4);
 #pragma unroll
-                    for (int k = 0; k < GEMM_BK / 16; ++k)
-                        tc_mma_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
-                    tc_commit_warp(&empty[s]);
+                    for (int k = 0; k < GEMM_BK / 16; ++k) {
+                        if constexpr (PAIR) tc_mma_pair_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
+                        else tc_mma_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
+                    }
+                    if constexpr (PAIR) tc_commit_pair_warp(&empty[s]);
+                    else tc_commit_warp(&empty[s]);
                 }
-                tc_commit_warp(&acc_full[buf]);
+                if constexpr (PAIR) tc_commit_pair_warp(&acc_full[buf]);
+                else tc_commit_warp(&acc_full[buf]);
             }
         }
     } else {
-        // ---------------------------------------------------------- epilogue
+        // ---------------------------------------------------------- epilogue (warps 2..9)
         // Warp ew = warp - 2 owns TMEM lane quadrant q (rows q*32 .. q*32+31 of
         // the tile; thread = row) and column half `half`, in 32-column blocks.
-        constexpr bool RES = EPI == EPI_RESID_GATE || EPI == EPI_RESID_CACHE;
-        constexpr bool CACHE = EPI == EPI_RESID_CACHE;
-        constexpr bool SHARED = epi_shared<EPI, BN>();
+        using E = EpiRing<BN, EPI, DEEP>;
         const int ew = warp - 2;
         const int q = warp & 3;
         const int half = ew >> 2;
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-        uint8_t *eb = smem + G::OFF_EPI + ew * epi_blocks<EPI, BN>() * EPI_BLOCK_BYTES;
-        uint8_t *s_out0 = eb;
-        uint8_t *s_aux = eb + EPI_BLOCK_BYTES;          // r_hat (cache) / resid (gate) / second out
-        uint8_t *s_res = (CACHE && !SHARED) ? eb + 2 * EPI_BLOCK_BYTES : (SHARED ? s_out0 : s_aux);
-        uint8_t *s_xin = SHARED ? s_aux : eb + 3 * EPI_BLOCK_BYTES;
-        uint64_t *lb = &ld_bar[ew];
-        const bool has_rhat = CACHE && ep.rhat != nullptr;
-        const uint32_t ld_bytes = (uint32_t)EPI_BLOCK_BYTES * (has_rhat ? 2u : 1u);
-        uint32_t n_ld = 0;                               // TMA loads issued on lb (its phases)
-        int n_st = 0;                                    // staging blocks written (out double-buffering)
-        auto load_res = [&](int m0, int col) {           // resid (+ x_in) block -> shared memory
-            if (lane == 0) {
-                mbar_expect_tx(lb, ld_bytes);
-                tma_load_2d(s_res, &em.resid, lb, col, m0 + q * 32);
-                if (has_rhat) tma_load_2d(s_xin, &em.xin, lb, col, m0 + q * 32);
+        uint8_t *eb = smem + G::OFF_EPI + ew * E::SLOTS * E::SLOT_BYTES;
+        float *vec = reinterpret_cast<float *>(smem + G::OFF_VEC) + ew * 64;     // bias [32], gate [32]
+        uint64_t *lb = ld_bar + ew * E::SLOTS;
+        const bool has_rhat = E::CACHE && ep.rhat != nullptr;
+        const int roff = row_off + q * 32;
+        int n = 0, n_ld = 0;                             // blocks done, residual loads issued
+        auto load_res = [&](int m, int col) {            // lane 0: residual operands of block n_ld
+            if constexpr (E::RES) {
+                uint8_t *s = eb + (n_ld % E::SLOTS) * E::SLOT_BYTES;
+                uint64_t *b = &lb[n_ld % E::SLOTS];
+                mbar_expect_tx(b, (uint32_t)EPI_BLOCK_BYTES * (has_rhat ? 2u : 1u));
+                tma_load_2d(s, &em.resid, b, col, m);
+                if (has_rhat) tma_load_2d(s + EPI_BLOCK_BYTES, &em.xin, b, col, m);
             }
-            ++n_ld;
         };
-        int local = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++local) {
+        Tile nt{0, 0, BN};                               // the next tile
+        if (worker < tw.n_items) {
+            nt = tile_at<G::BM, BN>(tw, worker);
+            if constexpr (E::RES)
+                for (; n_ld < E::AHEAD; ++n_ld)
+                    if (lane == 0) load_res(nt.m0 + roff, nt.n0 + half * (nt.w / 2) + 32 * n_ld);
+        }
+        int local = 0;
+        for (int item = worker; ok && item < tw.n_items; item += n_workers, ++local) {
             const int buf = local & 1;
             const uint32_t use = (uint32_t)(local >> 1);
-            int mb, nb;
-            tile_mn(tile, tiles_m, tiles_n, mb, nb);
-            const int m0 = mb * GEMM_BM, n0 = nb * BN;
-            const int row = m0 + q * 32 + lane;
-            if constexpr (SHARED) {
-                if (lane == 0) bulk_wait_read<0>();
-                __syncwarp();
-            }
-            if constexpr (RES) load_res(m0, n0 + half * (BN / 2));
+            const int coff = half * (nt.w / 2), n_blk = nt.w / 64;   // this warp's columns, 32 at a time
+            const int m0 = nt.m0 + roff, c0 = nt.n0 + coff;
+            const bool more = item + n_workers < tw.n_items;
+            if (more) nt = tile_at<G::BM, BN>(tw, item + n_workers);
+            const int row = m0 + lane;
             // RoPE position of this thread's row (camera, frame, h, w), once per tile
             int pos0 = 0, pos1 = 0, pos2 = 0, pos3 = 0;
             if constexpr (EPI == EPI_QKV_ROPE) {
@@ -298,51 +391,74 @@ __global__ void __launch_bounds__(320, 1)
                 pos2 = tp.z;
                 pos3 = tp.w;
             }
-            // bias (and gate) of this thread's columns, one value per lane,
-            // fetched one 32-column block ahead and broadcast by shuffles
-            const int colw = n0 + half * (BN / 2);
-            float b_next = ep.bias[colw + lane];
+            // bias (and gate) of a block's columns: one value per lane, fetched
+            // a block ahead, read back by every lane from shared memory
+            float b_next = ep.bias[c0 + lane];
             float g_next = 0.0f;
-            if constexpr (RES) g_next = ep.gate[colw + lane];
+            if constexpr (E::RES) g_next = ep.gate[c0 + lane];
             ok = mbar_wait(&acc_full[buf], use & 1, err, ERR_WAIT_EPI);
             __syncwarp();
             if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll 1
-            for (int j = 0; j < BN / 64; ++j) {
-                const int c = half * (BN / 2) + 32 * j;
-                const int col = n0 + c;
-                const float b_cur = b_next, g_cur = g_next;
-                if (j + 1 < BN / 64) {
+            for (int j = 0; j < n_blk; ++j, ++n) {
+                const int col = c0 + 32 * j;
+                uint8_t *s_out = eb + (n % E::SLOTS) * E::SLOT_BYTES;
+                vec[lane] = b_next;
+                if constexpr (E::RES) vec[32 + lane] = g_next;
+                if (j + 1 < n_blk) {
                     b_next = ep.bias[col + 32 + lane];
-                    if constexpr (RES) g_next = ep.gate[col + 32 + lane];
+                    if constexpr (E::RES) g_next = ep.gate[col + 32 + lane];
+                }
+                if constexpr (E::RES) {
+                    // operands of block n + AHEAD, into the slot whose last
+                    // store (block n + AHEAD - SLOTS) has been read
+                    const int ja = j + E::AHEAD;
+                    if (ja < n_blk || more) {
+                        if (lane == 0) {
+                            bulk_wait_read<E::SLOTS - E::AHEAD - 1>();
+                            if (ja < n_blk) load_res(m0, c0 + 32 * ja);
+                            else load_res(nt.m0 + roff, nt.n0 + half * (nt.w / 2) + 32 * (ja - n_blk));
+                        }
+                        ++n_ld;
+                    }
+                } else {
+                    if (lane == 0) bulk_wait_read<E::SLOTS - 1>();     // the slot's last store (block n - SLOTS) has been read
                 }
                 float v[32];
-                tmem_ld32_sync(tq + buf * BN + c, v);
-                if (j == BN / 64 - 1) {
-                    // last TMEM read of this tile: hand the accumulator back
-                    tc_fence_before();
-                    mbar_arrive(&acc_empty[buf]);
+                tmem_ld32_sync(tq + buf * BN + coff + 32 * j, v);
+                if (j == n_blk - 1) tc_fence_before();
+                __syncwarp();
+                // last TMEM read of this tile: hand the accumulator back
+                if (j == n_blk - 1 && lane == 0) {
+                    if constexpr (PAIR) mbar_arrive_cluster(map_to_cta(&acc_empty[buf], 0));
+                    else mbar_arrive(&acc_empty[buf]);
                 }
 #pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] += __shfl_sync(0xffffffffu, b_cur, i);
+                for (int i = 0; i < 32; i += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4 *>(vec + i);
+                    add2(v[i], v[i + 1], b4.x, b4.y);
+                    add2(v[i + 2], v[i + 3], b4.z, b4.w);
+                }
                 float xi[32];
-                if constexpr (RES) {
-                    ok = mbar_wait(lb, (n_ld - 1) & 1, err, ERR_WAIT_EPI);
+                if constexpr (E::RES) {
+                    ok = mbar_wait(&lb[n % E::SLOTS], (n / E::SLOTS) & 1, err, ERR_WAIT_EPI);
                     __syncwarp();
                     if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
                     float r[32];
-                    read_row32(s_res, lane, r);
-                    if constexpr (CACHE)
-                        if (has_rhat) read_row32(s_xin, lane, xi);
+                    read_row32(s_out, lane, r);
+                    if constexpr (E::CACHE)
+                        if (has_rhat) read_row32(s_out + EPI_BLOCK_BYTES, lane, xi);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = r[i] + __shfl_sync(0xffffffffu, g_cur, i) * v[i];
-                    __syncwarp();                      // every lane has read the block
-                    if (!SHARED && j + 1 < BN / 64) load_res(m0, col + 32);
+                    for (int i = 0; i < 32; i += 4) {
+                        const float4 g4 = *reinterpret_cast<const float4 *>(vec + 32 + i);
+                        fma2(v[i], v[i + 1], g4.x, g4.y, r[i], r[i + 1]);
+                        fma2(v[i + 2], v[i + 3], g4.z, g4.w, r[i + 2], r[i + 3]);
+                    }
                 }
                 if constexpr (EPI == EPI_GELU) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = gelu_tanh_approx(v[i]);
+                    for (int i = 0; i < 32; i += 2) gelu_tanh_approx2(v[i], v[i + 1]);
                 }
                 int part = 0, cl = col;
                 if constexpr (EPI == EPI_QKV_ROPE) {
@@ -362,40 +478,29 @@ __global__ void __launch_bounds__(320, 1)
                         }
                     }
                 }
-                // staging: out is double-buffered unless the block also carries
-                // residual operands; a buffer is rewritten once the TMA store
-                // that used it has read it
-                uint8_t *s_out = (RES || (n_st & 1) == 0) ? s_out0 : s_aux;
-                if (lane == 0) {
-                    if constexpr (RES) bulk_wait_read<0>();
-                    else bulk_wait_read<1>();
-                }
-                __syncwarp();
                 write_row32(s_out, lane, v);
-                if constexpr (CACHE) {
+                if constexpr (E::CACHE) {
                     if (has_rhat) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) v[i] = round_to<bf16>(v[i]) - xi[i];
-                        write_row32(s_aux, lane, v);
+                        write_row32(s_out + EPI_BLOCK_BYTES, lane, v);
                     }
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_2d(&em.out[part], s_out, cl, m0 + q * 32);
-                    if constexpr (CACHE)
-                        if (has_rhat) tma_store_2d(&em.rhat, s_aux, col, m0 + q * 32);
+                    tma_store_2d(&em.out[part], s_out, cl, m0);
+                    if constexpr (E::CACHE)
+                        if (has_rhat) tma_store_2d(&em.rhat, s_out + EPI_BLOCK_BYTES, col, m0);
                     bulk_commit();
                 }
-                ++n_st;
-                if constexpr (SHARED) {
-                    if (j + 1 < BN / 64) {
-                        if (lane == 0) bulk_wait_read<0>();
-                        __syncwarp();
-                        load_res(m0, col + 32);
-                    }
-                }
             }
+        }
+        // residual loads still in flight when a wait ran out
+        if constexpr (E::RES) {
+            if (!ok && lane == 0)
+                for (int k = n_ld - E::SLOTS < 0 ? 0 : n_ld - E::SLOTS; k < n_ld; ++k)
+                    mbar_wait(&lb[k % E::SLOTS], (k / E::SLOTS) & 1, err, ERR_WAIT_EPI);
         }
         // every TMA store of this warp has completed before the CTA exits
         if (lane == 0) bulk_wait_all();
@@ -403,9 +508,11 @@ __global__ void __launch_bounds__(320, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();           // no MMA, commit or arrival of the pair still to come
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, G::TMEM_COLS);
+        if constexpr (PAIR) tmem_dealloc_pair(tmem, G::TMEM_COLS);
+        else tmem_dealloc(tmem, G::TMEM_COLS);
     }
 }
 
@@ -520,25 +627,76 @@ static int gemm_sm_count() {
     return n;
 }
 
-// Output tile width for an M x N GEMM.  128 when 128 x 256 tiles would leave
-// SMs idle.  Otherwise the persistent grid runs ceil(tiles / SMs) rounds of
-// tiles; a 128 x 256 tile costs about 1.75 times a 128 x 128 one (it reuses
-// each A tile for twice the columns), so 256 is taken when its rounds cost no
-// more than the 128-wide tiles' rounds.
-int gemm_tc_bn(int M, int N) {
-    if (N % 256 != 0) return 128;
-    const long m_tiles = (M + GEMM_BM - 1) / GEMM_BM, n_sm = gemm_sm_count();
-    if (m_tiles * (N / 256) < n_sm) return 128;
-    const long r256 = (m_tiles * (N / 256) + n_sm - 1) / n_sm;
-    const long r128 = (m_tiles * (N / 128) + n_sm - 1) / n_sm;
-    return 7 * r256 <= 4 * r128 ? 256 : 128;
+// CTA pairs resident at once (both CTAs of a pair sit on neighbouring SMs).
+template <int EPI, bool DEEP>
+static int pair_count() {
+    static int n = 0;
+    if (n == 0) {
+        using G = GemmTile<256, EPI, DEEP>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2 * (gemm_sm_count() / 2));
+        cfg.blockDim = dim3(GEMM_THREADS);
+        cfg.dynamicSmemBytes = G::SMEM_BYTES;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int k = 0;
+        if (cudaOccupancyMaxActiveClusters(&k, gemm_tc_kernel<256, EPI, DEEP>, &cfg) != cudaSuccess || k < 1) {
+            cudaGetLastError();
+            k = gemm_sm_count() / 2;
+        }
+        n = k < 1 ? 1 : k;
+    }
+    return n;
 }
 
-template <int EPI, int BN>
-static cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tb, const EpiParams &ep, int K,
+// Walk of a pair grid over 256 x 256 tiles: a remainder of at most half of
+// the pairs is cut into halves.
+static TileWalk pair_walk(int M, int N, int workers) {
+    TileWalk tw;
+    tw.tiles_m = (M + 255) / 256;
+    tw.tiles_n = N / 256;
+    const int n = tw.tiles_m * tw.tiles_n, rem = n % workers;
+    tw.n_full = 2 * rem <= workers ? n - rem : n;
+    tw.n_items = tw.n_full + 2 * (n - tw.n_full);
+    return tw;
+}
+
+// Output tiling for an M x N x K GEMM: 256 (CTA pairs), 128 or 64 (single
+// CTAs).  Half the pairs' worth of 256 x 256 tiles and fewer are one round of
+// single tiles, 64 wide while those find an SM each.  Beyond, the cost in SM
+// cycles of the persistent rounds: a 64-deep k step takes about 555 cycles
+// on a full pair tile, 340 on a half one, 450 on a single tile with every SM
+// busy (bound by its operand feed); no round is shorter than its epilogue,
+// the last one's is added, and setting up a pair takes some 1500 more.
+// Measured, pair / 128-wide single: 8064 x 512 x 512 8.5 / 7.6 us, 840 x 1024
+// x 256 7.3 / 4.6, 8064 x 2048 x 512 + GELU 16.6 / 18.1, 700 x 5120 x 1024 +
+// residual cache 17.6 / 14.3, 239 x 12032 x 3712 22.0 / 27.7, 1554 x 6144 x
+// 11072 142 / 176, 12960 x 5120 x 5120 366 / 498.
+int gemm_tc_bn(int epi, int M, int N, int K) {
+    const long n_sm = gemm_sm_count(), pairs = n_sm / 2 < 1 ? 1 : n_sm / 2;
+    const long t128 = (long)((M + 127) / 128) * (N / 128), r128 = (t128 + n_sm - 1) / n_sm;
+    if (2 * t128 <= n_sm) return 64;
+    if (N % 256 != 0) return 128;
+    const TileWalk tw = pair_walk(M, N, (int)pairs);
+    if (tw.n_full == 0) return 128;
+    const long r_full = (tw.n_full + pairs - 1) / pairs, r_half = tw.n_items > tw.n_full ? 1 : 0;
+    const long kt = K / GEMM_BK;
+    const long e_full = epi == EPI_RESID_CACHE ? 12000 : 4500, e_half = epi == EPI_RESID_CACHE ? 6000 : 2500;
+    const long pair = r_full * std::max(kt * 555, e_full) + r_half * std::max(kt * 340, e_half) +
+                      (r_half ? e_half : e_full) + 1500;
+    return pair <= r128 * std::max(kt * 450, e_half) + e_half ? 256 : 128;
+}
+
+template <int EPI, int BN, bool DEEP = false>
+static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                              const uint8_t *skip, int *err, cudaStream_t st) {
-    using G = GemmTile<BN, EPI>;
-    auto kern = gemm_tc_kernel<BN, EPI>;
+    using G = GemmTile<BN, EPI, DEEP>;
+    auto kern = gemm_tc_kernel<BN, EPI, DEEP>;
     EpiMaps em;
     if (!build_epi_maps<EPI>(em, ep)) return cudaErrorInvalidValue;
     static bool attr_set = false;
@@ -547,19 +705,31 @@ static cudaError_t launch_tc(const CUtensorMap &ta, const CUtensorMap &tb, const
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    const int n_sm = gemm_sm_count();
-    const int n_tiles = (ep.N / BN) * ((ep.M + GEMM_BM - 1) / GEMM_BM);
-    const int grid = n_tiles < n_sm ? n_tiles : n_sm;
-    return launch_pdl(kern, dim3(grid), dim3(320), G::SMEM_BYTES, st, ta, tb, em, ep, K, skip, err);
+    int workers = gemm_sm_count();
+    TileWalk tw;
+    if constexpr (G::PAIR) {
+        workers = pair_count<EPI, DEEP>();
+        tw = pair_walk(ep.M, ep.N, workers);
+    } else {
+        tw.tiles_m = (ep.M + GEMM_BM - 1) / GEMM_BM;
+        tw.tiles_n = ep.N / BN;
+        tw.n_full = tw.n_items = tw.tiles_m * tw.tiles_n;
+    }
+    if (tw.n_items < workers) workers = tw.n_items;
+    return launch_pdl_cluster(kern, G::PAIR ? 2 : 1, dim3(G::PAIR ? 2 * workers : workers), dim3(GEMM_THREADS), G::SMEM_BYTES, st,
+                              ta, tb, em, ep, K, tw, skip, err);
 }
 
 template <int BN>
-static cudaError_t gemm_tc_bn_(int epi, const CUtensorMap &ta, const CUtensorMap &tb, const EpiParams &ep, int K,
+static cudaError_t gemm_tc_bn_(int epi, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                                const uint8_t *skip, int *err, cudaStream_t st) {
     switch (epi) {
         case EPI_BIAS: return launch_tc<EPI_BIAS, BN>(ta, tb, ep, K, skip, err, st);
         case EPI_GELU: return launch_tc<EPI_GELU, BN>(ta, tb, ep, K, skip, err, st);
-        case EPI_RESID_GATE: return launch_tc<EPI_RESID_GATE, BN>(ta, tb, ep, K, skip, err, st);
+        case EPI_RESID_GATE:
+            if constexpr (BN == 64) return launch_tc<EPI_RESID_GATE, BN>(ta, tb, ep, K, skip, err, st);
+            return K < 1536 ? launch_tc<EPI_RESID_GATE, BN, true>(ta, tb, ep, K, skip, err, st)
+                            : launch_tc<EPI_RESID_GATE, BN>(ta, tb, ep, K, skip, err, st);
         case EPI_RESID_CACHE: return launch_tc<EPI_RESID_CACHE, BN>(ta, tb, ep, K, skip, err, st);
         case EPI_QKV_ROPE: return launch_tc<EPI_QKV_ROPE, BN>(ta, tb, ep, K, skip, err, st);
         default: return cudaErrorInvalidValue;
@@ -567,12 +737,13 @@ static cudaError_t gemm_tc_bn_(int epi, const CUtensorMap &ta, const CUtensorMap
 }
 
 // Entry used by the chunk step and xc_op_linear / xc_op_qkv_rope (bf16 only).
-// `ta` covers A [M][K] (box 128 rows), `tb` covers Wt [N][K] with box rows
-// = bn (gemm_tc_bn(M, N)); N % bn == 0, K % 64 == 0.
-cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const CUtensorMap &tb, const EpiParams &ep, int K,
+// `ta` covers A [M][K] (boxes of 128 rows), `tb` Wt [N][K]; bn =
+// gemm_tc_bn(epi, M, N, K); N % bn == 0, K % 64 == 0.
+cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                     const uint8_t *skip, int *err, cudaStream_t st) {
     if (bn == 256) return gemm_tc_bn_<256>(epi, ta, tb, ep, K, skip, err, st);
     if (bn == 128) return gemm_tc_bn_<128>(epi, ta, tb, ep, K, skip, err, st);
+    if (bn == 64) return gemm_tc_bn_<64>(epi, ta, tb, ep, K, skip, err, st);
     return cudaErrorInvalidValue;
 }
 

@@ -217,9 +217,11 @@ struct xc_ctx {
 
     // tensor maps (bf16); output tile width of each GEMM
     CUtensorMap tm_h, tm_o, tm_u, tm_q;
-    int bn_qkv, bn_o, bn_f1, bn_f2;
-    std::vector<CUtensorMap> tm_wqkv, tm_wo, tm_w1, tm_w2, tm_rk, tm_rv;
-    std::vector<CUtensorMap> tm_caq, tm_cao, tm_cak, tm_cav, tm_ck, tm_cv;   // cross-attention
+    int bn_qkv, bn_o, bn_f1, bn_f2, bn_caq;
+    std::vector<WeightMaps> tm_wqkv, tm_wo, tm_w1, tm_w2;
+    std::vector<CUtensorMap> tm_rk, tm_rv;
+    std::vector<WeightMaps> tm_caq, tm_cao, tm_cak, tm_cav;                  // cross-attention
+    std::vector<CUtensorMap> tm_ck, tm_cv;
 
     int n, next_step;
     void *trace;
@@ -448,6 +450,11 @@ void tmap(xc_ctx *ctx, CUtensorMap *m, const void *base, uint64_t rows, uint64_t
                 (unsigned long long)cols);
         throw Fail{XC_ECUDA};
     }
+}
+
+void wmap(xc_ctx *ctx, WeightMaps *m, const void *base, uint64_t rows, uint64_t cols) {
+    tmap(ctx, &m->box128, base, rows, cols, 128);
+    tmap(ctx, &m->box64, base, rows, cols, 64);
 }
 
 // Profiling hooks: an event pair around one launch when its kind is selected.
@@ -728,7 +735,7 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
             ep.out = qb;
             if constexpr (sizeof(T) == 2) {
                 LAUNCH(XC_K_XATTN, b, 1,
-                       gemm_tc(EPI_BIAS, ctx->bn_o, ctx->tm_h, ctx->tm_caq[b], ep, d, flag, ctx->d_err, st));
+                       gemm_tc(EPI_BIAS, ctx->bn_caq, ctx->tm_h, ctx->tm_caq[b], ep, d, flag, ctx->d_err, st));
                 int n_x = 1;
                 LAUNCH(XC_K_XATTN, b, n_x,
                        attn_tc(hd, ctx->tm_q, ctx->tm_ck[b], ctx->tm_cv[b], reinterpret_cast<bf16 *>(ob), L,
@@ -1117,10 +1124,11 @@ xc_status xc_init(const xc_model_cfg *cfg, const xc_weights *w, void *cuda_strea
 
         // tensor maps of the bf16 path
         if (ctx->bf) {
-            ctx->bn_qkv = gemm_tc_bn(L, 3 * d);
-            ctx->bn_o = gemm_tc_bn(L, d);
-            ctx->bn_f1 = gemm_tc_bn(L, F);
-            ctx->bn_f2 = gemm_tc_bn(L, d);
+            ctx->bn_qkv = gemm_tc_bn(EPI_QKV_ROPE, L, 3 * d, d);
+            ctx->bn_o = gemm_tc_bn(EPI_RESID_GATE, L, d, d);
+            ctx->bn_caq = gemm_tc_bn(EPI_BIAS, L, d, d);
+            ctx->bn_f1 = gemm_tc_bn(EPI_GELU, L, F, d);
+            ctx->bn_f2 = gemm_tc_bn(EPI_RESID_CACHE, L, d, F);
             tmap(ctx, &ctx->tm_h, ctx->hbuf, L, d, 128);
             tmap(ctx, &ctx->tm_o, ctx->o, L, d, 128);
             tmap(ctx, &ctx->tm_u, ctx->u, L, F, 128);
@@ -1136,10 +1144,10 @@ xc_status xc_init(const xc_model_cfg *cfg, const xc_weights *w, void *cuda_strea
                 const char *wo = reinterpret_cast<const char *>(ctx->o_wt) + (size_t)b * d * d * es;
                 const char *w1 = reinterpret_cast<const char *>(ctx->f1_wt) + (size_t)b * F * d * es;
                 const char *w2 = reinterpret_cast<const char *>(ctx->f2_wt) + (size_t)b * d * F * es;
-                tmap(ctx, &ctx->tm_wqkv[b], wq, 3 * (uint64_t)d, d, ctx->bn_qkv);
-                tmap(ctx, &ctx->tm_wo[b], wo, d, d, ctx->bn_o);
-                tmap(ctx, &ctx->tm_w1[b], w1, F, d, ctx->bn_f1);
-                tmap(ctx, &ctx->tm_w2[b], w2, d, F, ctx->bn_f2);
+                wmap(ctx, &ctx->tm_wqkv[b], wq, 3 * (uint64_t)d, d);
+                wmap(ctx, &ctx->tm_wo[b], wo, d, d);
+                wmap(ctx, &ctx->tm_w1[b], w1, F, d);
+                wmap(ctx, &ctx->tm_w2[b], w2, d, F);
                 const char *rk = reinterpret_cast<const char *>(ctx->ring_k) + (size_t)b * ctx->Wkv * Ld * es;
                 const char *rv = reinterpret_cast<const char *>(ctx->ring_v) + (size_t)b * ctx->Wkv * Ld * es;
                 tmap(ctx, &ctx->tm_rk[b], rk, (uint64_t)ctx->Wkv * L, d, 128);
@@ -1147,16 +1155,16 @@ xc_status xc_init(const xc_model_cfg *cfg, const xc_weights *w, void *cuda_strea
             }
             if (ctx->xattn) {
                 const int D = ctx->d_ctx;
-                for (auto *v : {&ctx->tm_caq, &ctx->tm_cao, &ctx->tm_cak, &ctx->tm_cav, &ctx->tm_ck, &ctx->tm_cv})
-                    v->resize(B);
+                for (auto *v : {&ctx->tm_caq, &ctx->tm_cao, &ctx->tm_cak, &ctx->tm_cav}) v->resize(B);
+                for (auto *v : {&ctx->tm_ck, &ctx->tm_cv}) v->resize(B);
                 for (int b = 0; b < B; ++b) {
                     const char *wq = reinterpret_cast<const char *>(ctx->ca_q_wt) + (size_t)b * d * d * es;
                     const char *wo = reinterpret_cast<const char *>(ctx->ca_o_wt) + (size_t)b * d * d * es;
                     const char *wkv = reinterpret_cast<const char *>(ctx->ca_kv_wt) + (size_t)b * 2 * d * D * es;
-                    tmap(ctx, &ctx->tm_caq[b], wq, d, d, ctx->bn_o);
-                    tmap(ctx, &ctx->tm_cao[b], wo, d, d, ctx->bn_o);
-                    tmap(ctx, &ctx->tm_cak[b], wkv, d, D, 128);                      // rows [0, d): W_k^T
-                    tmap(ctx, &ctx->tm_cav[b], wkv + (size_t)d * D * es, d, D, 128);  // rows [d, 2d): W_v^T
+                    wmap(ctx, &ctx->tm_caq[b], wq, d, d);
+                    wmap(ctx, &ctx->tm_cao[b], wo, d, d);
+                    wmap(ctx, &ctx->tm_cak[b], wkv, d, D);                      // rows [0, d): W_k^T
+                    wmap(ctx, &ctx->tm_cav[b], wkv + (size_t)d * D * es, d, D);  // rows [d, 2d): W_v^T
                     const size_t cb = (size_t)b * ctx->max_ctx * d * es;
                     tmap(ctx, &ctx->tm_ck[b], reinterpret_cast<const char *>(ctx->ctx_k) + cb, ctx->max_ctx, d, 128);
                     tmap(ctx, &ctx->tm_cv[b], reinterpret_cast<const char *>(ctx->ctx_v) + cb, ctx->max_ctx, d, 128);
@@ -1375,7 +1383,7 @@ xc_status xc_set_context(xc_ctx *ctx, const float *context, int n_ctx) {
                 ep.out = reinterpret_cast<char *>(half ? ctx->ctx_v : ctx->ctx_k) +
                          (size_t)b * ctx->max_ctx * d * ctx->esz;
                 if (ctx->bf) {
-                    CK(gemm_tc(EPI_BIAS, 128, tm_a, half ? ctx->tm_cav[b] : ctx->tm_cak[b], ep, D, nullptr,
+                    CK(gemm_tc(EPI_BIAS, gemm_tc_bn(EPI_BIAS, n_ctx, d, D), tm_a, half ? ctx->tm_cav[b] : ctx->tm_cak[b], ep, D, nullptr,
                                ctx->d_err, st));
                 } else {
                     const float *W = reinterpret_cast<const float *>(ctx->ca_kv_wt) + ((size_t)b * 2 + half) * d * D;
@@ -1554,9 +1562,10 @@ xc_status xc_op_linear(int dtype, int epilogue, int M, int N, int K, const void 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (dtype == XC_BF16) {
         if (N % 256 != 0 || K % 64 != 0) OP_FAIL(XC_EINVAL, "xc_op_linear: bf16 needs N %% 256 == 0, K %% 64 == 0");
-        CUtensorMap ta, tb;
-        const int bn = gemm_tc_bn(M, N);
-        if (!make_tmap_bf16(&ta, A, M, K, 128) || !make_tmap_bf16(&tb, Wt, N, K, bn))
+        CUtensorMap ta;
+        WeightMaps tb;
+        const int bn = gemm_tc_bn(epilogue, M, N, K);
+        if (!make_tmap_bf16(&ta, A, M, K, 128) || !make_weight_maps(&tb, Wt, N, K))
             OP_FAIL(XC_EINVAL, "xc_op_linear: tensor map (alignment?)");
         OP_CK(gemm_tc(epilogue, bn, ta, tb, ep, K, nullptr, op_err_word(), st));
     } else if (dtype == XC_F32) {
@@ -1618,9 +1627,10 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
     cudaStream_t st = st0;
     if (dtype == XC_BF16) {
         if ((3 * d) % 256 != 0 || d % 64 != 0) OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: bf16 needs 3d %% 256, d %% 64");
-        CUtensorMap ta, tb;
-        const int bn = gemm_tc_bn(M, 3 * d);
-        if (!make_tmap_bf16(&ta, A, M, d, 128) || !make_tmap_bf16(&tb, Wt, 3 * (uint64_t)d, d, bn))
+        CUtensorMap ta;
+        WeightMaps tb;
+        const int bn = gemm_tc_bn(EPI_QKV_ROPE, M, 3 * d, d);
+        if (!make_tmap_bf16(&ta, A, M, d, 128) || !make_weight_maps(&tb, Wt, 3 * (uint64_t)d, d))
             OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: tensor map");
         OP_CK(gemm_tc(EPI_QKV_ROPE, bn, ta, tb, ep, d, nullptr, op_err_word(), st));
     } else if (dtype == XC_F32) {

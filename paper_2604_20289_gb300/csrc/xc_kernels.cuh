@@ -87,8 +87,16 @@ template <typename T>
 cudaError_t chain_apply(T *x0, T *x1, const T *rhat_t, const uint8_t *flags, int b, int n_blocks, long ld,
                         int n_sm, cudaStream_t st);
 bool make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows);
-int gemm_tc_bn(int M, int N);
-cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const CUtensorMap &tb, const EpiParams &ep, int K,
+// A weight matrix Wt [N][K] of the bf16 GEMM, in boxes of 128 rows and, for
+// the half tiles of a last round, of 64.
+struct WeightMaps {
+    CUtensorMap box128, box64;
+};
+inline bool make_weight_maps(WeightMaps *m, const void *base, uint64_t N, uint64_t K) {
+    return make_tmap_bf16(&m->box128, base, N, K, 128) && make_tmap_bf16(&m->box64, base, N, K, 64);
+}
+int gemm_tc_bn(int epi, int M, int N, int K);
+cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                     const uint8_t *skip, int *err, cudaStream_t st);
 cudaError_t attn_tc(int head_dim, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, bf16 *o,
                     int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes, const uint8_t *skip, int *err,

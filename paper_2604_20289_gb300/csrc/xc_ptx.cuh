@@ -59,12 +59,74 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *e
     return false;
 }
 
+// ------------------------------------------------------------------ CTA pair
+// Two CTAs of a cluster of 2 that share tcgen05.mma.cta_group::2 tiles.
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// shared::cluster address of the same offset in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t map_to_cta(const void *p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+// Arrival on a barrier of either CTA.  Release at CTA scope only: what it hands
+// over is tensor memory already read (tcgen05.wait::ld), and a cluster-scope
+// release waits for every outstanding memory operation of the thread (2500 to
+// 7000 cycles per output tile in the GEMM epilogue).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// Every thread of both CTAs (a hardware barrier: both reach it on every path).
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // ----------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *tm, uint64_t *bar, int x, int y) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(smem_u32(bar))
         : "memory");
+}
+// One stage of two tiles: `bytes` expected on `bar` and both loads issued, by
+// one elected lane of a converged warp.
+__device__ __forceinline__ void tma_stage_warp(uint64_t *bar, uint32_t bytes, void *dst_a, const CUtensorMap *tm_a,
+                                               int ya, void *dst_b, const CUtensorMap *tm_b, int yb, int x) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
+        "elect.sync r|e, 0xffffffff;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%8, %4}], [%0];\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%5], [%6, {%8, %7}], [%0];\n\t}"
+        ::"r"(smem_u32(bar)), "r"(bytes), "r"(smem_u32(dst_a)), "l"(reinterpret_cast<uint64_t>(tm_a)), "r"(ya),
+        "r"(smem_u32(dst_b)), "l"(reinterpret_cast<uint64_t>(tm_b)), "r"(yb), "r"(x)
+        : "memory");
+}
+// The same for a CTA pair: the bytes are counted on a barrier of the leader
+// (`cluster_bar`, its shared::cluster address) and expected there, for both
+// CTAs, by the leader alone (`bar` its local address, `lead` != 0).  The
+// peer's bytes may arrive before the leader's expect_tx of the same phase: the
+// phase cannot complete without the leader's arrival.
+__device__ __forceinline__ void tma_stage_pair_warp(uint64_t *bar, uint32_t cluster_bar, uint32_t lead, uint32_t bytes,
+                                                    void *dst_a, const CUtensorMap *tm_a, int ya, void *dst_b,
+                                                    const CUtensorMap *tm_b, int yb, int x) {
+    asm volatile(
+        "{\n\t.reg .pred e, l;\n\t.reg .b32 r;\n\t"
+        "elect.sync r|e, 0xffffffff;\n\t"
+        "setp.ne.and.u32 l, %10, 0, e;\n\t"
+        "@l mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t"
+        "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%8, %4}], [%9];\n\t"
+        "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%5], [%6, {%8, %7}], [%9];\n\t}"
+        ::"r"(smem_u32(bar)), "r"(bytes), "r"(smem_u32(dst_a)), "l"(reinterpret_cast<uint64_t>(tm_a)), "r"(ya),
+        "r"(smem_u32(dst_b)), "l"(reinterpret_cast<uint64_t>(tm_b)), "r"(yb), "r"(x), "r"(cluster_bar), "r"(lead)
+        : "memory");
+}
+// Fetches the descriptor ahead of its first copy.
+__device__ __forceinline__ void prefetch_tmap(const CUtensorMap *tm) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
 }
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -80,6 +142,16 @@ __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// CTA pair: one warp of each CTA makes the call.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t *slot, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -135,6 +207,29 @@ __device__ __forceinline__ void tc_commit_warp(uint64_t *bar) {
         "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t"
         "elect.sync r|e, 0xffffffff;\n\t"
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        ::"r"(smem_u32(bar))
+        : "memory");
+}
+// CTA pair, issued by the leader's warp: M = 256 over both CTAs (each supplies
+// 128 rows of A and half of B's rows from its own shared memory, at the same
+// offsets, and accumulates its 128 rows in its own TMEM).
+__device__ __forceinline__ void tc_mma_pair_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred e, p;\n\t.reg .b32 r;\n\t"
+        "elect.sync r|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Arrives on the barrier at this offset in both CTAs of the pair.
+__device__ __forceinline__ void tc_commit_pair_warp(uint64_t *bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t.reg .b32 r;\n\t.reg .b16 m;\n\t"
+        "elect.sync r|e, 0xffffffff;\n\t"
+        "mov.b16 m, 3;\n\t"
+        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n\t}"
         ::"r"(smem_u32(bar))
         : "memory");
 }
