@@ -25,10 +25,12 @@
 // At head_dim 64 the two softmax warps of each SM sub-partition (one per
 // tile) take turns on the MUFU-bound exponential phase.
 // Online softmax in the exp2 domain with lazy rescaling: a row's O and sum
-// are rescaled only when its running max grows by more than 8 (2^8 headroom
-// in fp32 / bf16).  Score scaling and row sums use packed fp32 pairs
+// are rescaled only when its running max grows by more than 8 (hd 64), or
+// when a tile's row sum passes 2^40 under the max in use (hd 128).  Score scaling and row sums use packed fp32 pairs
 // (FFMA2 / FADD2).  Keys beyond n_keys (ragged last tile) are masked to -inf;
 // their K/V rows are finite (zero-initialised ring, TMA zero fill).
+#include <algorithm>
+
 #include "xc_ptx.cuh"
 
 namespace xc {
@@ -43,7 +45,8 @@ struct AttnTile {
     static constexpr int STAGES = HD == 64 ? 4 : 2;
     static constexpr int OFF_K = QT * Q_BYTES;
     static constexpr int OFF_V = OFF_K + STAGES * KV_BYTES;
-    static constexpr int OFF_BAR = OFF_V + STAGES * KV_BYTES;
+    static constexpr int OFF_O = OFF_V + STAGES * KV_BYTES;    // output staging, 4 KB per softmax warp
+    static constexpr int OFF_BAR = OFF_O + 8 * 4096;
     static constexpr int SMEM_BYTES = OFF_BAR + 512 + 1024;
     static constexpr int TMEM_COLS = 512;
     static constexpr int THREADS = 352;            // 8 softmax, 1 TMA, 2 MMA warps
@@ -52,7 +55,8 @@ struct AttnTile {
     __host__ __device__ static constexpr int S_COL(int i) { return 128 * i; }
     __host__ __device__ static constexpr int O_COL(int i) { return 256 + HD * i; }
     __host__ __device__ static constexpr int P_COL(int i) { return SEP_P ? 256 + 2 * HD + 64 * i : 128 * i; }
-    static constexpr float LAZY = 8.0f;                // rescale threshold (log2 units)
+    static constexpr float LAZY = 8.0f;                // hd 64: rescale threshold (log2 units)
+    static constexpr float RAISE = 1099511627776.0f;   // hd 128: 2^40, a tile's row sum
 };
 
 __device__ __forceinline__ uint8_t *align1024_a(uint8_t *p) {
@@ -66,15 +70,56 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return y;
 }
 
+// Max of a 128-column score row: 16 independent chains of three-input max over
+// columns 0..111, the last 16 columns, then a tree.
+__device__ __forceinline__ float row_max(const float (&s)[128]) {
+    float mx[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) mx[k] = s[k];
+#pragma unroll
+    for (int c = 16; c < 112; c += 32) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) mx[k] = fmax3(mx[k], s[c + k], s[c + 16 + k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) mx[k] = fmaxf(mx[k], s[112 + k]);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) mx[k] = fmax3(mx[k], mx[k + 5], mx[k + 10]);
+    return fmax3(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[15]), mx[0]);
+}
+
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
+// Probabilities 2^(s * sl2 - m) of the 32 scores of quarter qt, packed to bf16
+// pairs and stored to TMEM; their sums go to rs0, rs1.
+__device__ __forceinline__ void exp_quarter(const float (&s)[128], int qt, float sl2, float m, uint32_t tP,
+                                            float2 &rs0, float2 &rs1) {
+    const float2 sc2 = make_float2(sl2, sl2), nm2 = make_float2(-m, -m);
+    uint32_t w[16];
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+        const int c = 32 * qt + 2 * k;
+        const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), sc2, nm2);
+        const float2 b = __ffma2_rn(make_float2(s[c + 2], s[c + 3]), sc2, nm2);
+        const float2 pa = make_float2(ex2_approx(a.x), ex2_approx(a.y));
+        const float2 pb = make_float2(ex2_approx(b.x), ex2_approx(b.y));
+        rs0 = __fadd2_rn(rs0, pa);
+        rs1 = __fadd2_rn(rs1, pb);
+        __nv_bfloat162 h0 = __floats2bfloat162_rn(pa.x, pa.y);
+        __nv_bfloat162 h1 = __floats2bfloat162_rn(pb.x, pb.y);
+        w[k] = *reinterpret_cast<uint32_t *>(&h0);
+        w[k + 1] = *reinterpret_cast<uint32_t *>(&h1);
+    }
+    tmem_st16u_sync(tP + 16 * qt, w);
+}
+
 // Work split.  A unit is (head, pair of 128-query tiles), u = head * n_qblk +
-// qblk, with n_kt key tiles.  Without a split (G = n_units CTAs) every CTA
-// runs one whole unit.  With G = number of SMs < n_units, two orders:
+// qblk, with n_kt key tiles, walked by G CTAs (one per SM) in one of two
+// orders:
 //  * contiguous (WAVE = false): the (unit, key tile) iteration space, T =
 //    n_units * n_kt, is cut into the contiguous shares [c T / G,
 //    (c + 1) T / G).  A unit cut by the boundary between CTAs c - 1 and c is
@@ -84,21 +129,22 @@ __device__ __forceinline__ float ex2_approx(float x) {
 //    unit, so a unit is cut at most once.  The units in flight span every
 //    head, so each unit streams its head's K / V from DRAM once the heads'
 //    K / V exceed L2.
-//  * waves (WAVE = true, for many waves of units whose K / V exceed L2):
-//    W = n_units / G waves of whole units -- CTA c runs units c, c + G, ...,
-//    c + (W - 1) G, so the CTAs running at one time share a few heads and
-//    each K / V tile comes from DRAM once per wave -- then the R = n_units -
-//    W G remaining units, T2 = R n_kt key tiles, are split evenly: CTA c
-//    takes [c T2 / G, (c + 1) T2 / G), less than one unit, touching at most
-//    two units (its pieces W and W + 1, partial slots 2 c and 2 c + 1),
-//    merged per remaining unit by attn_combine_kernel.
+//  * waves (WAVE = true): CTA c runs the whole units c, c + G, ..., W of
+//    them and one more if c < R -- the CTAs running at one time share a few
+//    heads and each K / V tile comes from DRAM once per wave -- and, where
+//    T2 > 0 (then R = 0), the key tiles of the remaining units, T2 of them,
+//    are split evenly: CTA c takes [c T2 / G, (c + 1) T2 / G), at most one
+//    unit's worth, touching at most two units (its pieces W and W + 1,
+//    partial slots 2 c and 2 c + 1), merged per remaining unit by
+//    attn_combine_kernel.  With fewer units than SMs W = 0: every unit is
+//    such a remaining one.
 // Each role walks the CTA's key tiles with a cursor (TileCursor): tile
 // counter g, unit u and its key tile k; in the wave order also the piece
 // index p and the unit step du.
 struct AttnSplit {
     long long T;          // contiguous: total iterations
-    long long T2;         // waves: key tiles of the remaining units
-    int n_kt, n_qblk, G, W;
+    long long T2;         // waves: key tiles of the remaining units, split evenly
+    int n_kt, n_qblk, G, W, R;
     __host__ __device__ long long begin(int c) const { return T * c / G; }
     __host__ __device__ long long begin2(int c) const { return T2 * c / G; }
 };
@@ -125,11 +171,25 @@ __device__ __forceinline__ RemSeg rem_seg(const AttnSplit &sp, int c) {
     return r;
 }
 
+// Partials: slot sl's O as 4 KB blocks [softmax warp 0..7][32-column group][32
+// rows][32 fp32], the 16-byte chunks of a row permuted by its row number (so
+// that a lane writes its row to shared memory without bank conflicts and the
+// block leaves as one bulk copy).
+__host__ __device__ constexpr size_t partial_block(int slot, int warp, int grp, int hd) {
+    return ((size_t)(slot * 8 + warp) * (hd / 32) + grp) * 1024;
+}
+
+__device__ __forceinline__ void bulk_store(void *dst, const void *src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)),
+                 "r"(smem_u32(src)), "r"(bytes)
+                 : "memory");
+}
+
 template <int HD, bool WAVE>
 __global__ void __launch_bounds__(352, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const __grid_constant__ CUtensorMap tmV, bf16 *__restrict__ o, const int Lq,
-                   const int n_keys, const int d, const AttnSplit sp, float *__restrict__ ws_o,
+                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const int Lq,
+                   const int n_keys, const AttnSplit sp, float *__restrict__ ws_o,
                    float2 *__restrict__ ws_ml, const uint8_t *__restrict__ skip_flag, int *err) {
     pdl_wait();
     using A = AttnTile<HD>;
@@ -159,8 +219,9 @@ __global__ void __launch_bounds__(352, 1)
     const int cta = blockIdx.x;
     long long it0 = 0;
     int n_t;                                       // key tiles of this CTA (>= 1)
+    const int n_whole = sp.W + (cta < sp.R ? 1 : 0);   // waves: whole units of this CTA
     if constexpr (WAVE) {
-        n_t = sp.W * nkt + (int)(sp.begin2(cta + 1) - sp.begin2(cta));
+        n_t = n_whole * nkt + (int)(sp.begin2(cta + 1) - sp.begin2(cta));
     } else {
         it0 = sp.begin(cta);
         n_t = (int)(sp.begin(cta + 1) - it0);
@@ -172,9 +233,9 @@ __global__ void __launch_bounds__(352, 1)
     // to the remainder at tile gw, so the per-tile tests stay the same.
     RemSeg rem{0, 0, 0, 0};
     if constexpr (WAVE) rem = rem_seg(sp, cta);
-    const int gw = WAVE ? sp.W * nkt : -1;
+    const int gw = WAVE ? n_whole * nkt : -1;
     TileCursor c0{0, u0, (int)(it0 % nkt), 0, 1};
-    if constexpr (WAVE) c0 = sp.W > 0 ? TileCursor{0, cta, 0, 0, sp.G} : TileCursor{0, rem.u, rem.k0, 0, 1};
+    if constexpr (WAVE) c0 = n_whole > 0 ? TileCursor{0, cta, 0, 0, sp.G} : TileCursor{0, rem.u, rem.k0, 0, 1};
     auto piece_of = [&](const TileCursor &c) {    // index of the cursor's piece in this CTA
         if constexpr (WAVE) return c.p;
         else return c.u - u0;
@@ -417,36 +478,8 @@ __global__ void __launch_bounds__(352, 1)
                 for (int c = 0; c < 128; ++c)
                     if (c >= tail) s[c] = -INFINITY;
             }
-            // row max: 16 independent chains of three-input max over columns
-            // 0..111, the last 16 columns, then a tree
-            float mx[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) mx[k] = s[k];
-#pragma unroll
-            for (int c = 16; c < 112; c += 32) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) mx[k] = fmax3(mx[k], s[c + k], s[c + 16 + k]);
-            }
-#pragma unroll
-            for (int k = 0; k < 16; ++k) mx[k] = fmaxf(mx[k], s[112 + k]);
-#pragma unroll
-            for (int k = 0; k < 5; ++k) mx[k] = fmax3(mx[k], mx[k + 5], mx[k + 10]);
-            const float m_new = fmax3(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[15]), mx[0]) * sl2;
-            if (fresh) m = m_new;
-            const bool grow = !fresh && m_new > m + A::LAZY;
-            const float alpha = grow ? ex2_approx(m - m_new) : 1.0f;
-            if (grow) m = m_new;
-            if constexpr (A::SEP_P) {
-                // P_i buffer free and O_i stable once P V of the previous tile is done
-                if (g >= 1) {
-                    ok = mbar_wait(&pv_done[wg], (g - 1) & 1, err, ERR_WAIT_SOFTMAX);
-                    __syncwarp();
-                    if (!__all_sync(0xffffffffu, ok)) return false;
-                    tc_fence_after();
-                }
-            }
-            // (hd 128: the commit behind s_full already covers P V of tile g-1)
-            if (__any_sync(0xffffffffu, grow)) {
+            // O_i (this thread's row of it, in TMEM) times alpha; the whole warp
+            auto scale_o = [&](float alpha) {
 #pragma unroll 1
                 for (int c = 0; c < HD / 16; ++c) {
                     float t[16];
@@ -455,7 +488,59 @@ __global__ void __launch_bounds__(352, 1)
                     for (int i = 0; i < 16; ++i) t[i] *= alpha;
                     tmem_st16_sync(tO + 16 * c, t);
                 }
+            };
+            float2 rs0 = make_float2(0.f, 0.f), rs1 = make_float2(0.f, 0.f);
+            if constexpr (!A::SEP_P) {
+                // hd 128.  m is the row max of the piece's first tile; a later
+                // tile takes it as it is, without a max of its own: bf16 and
+                // fp32 share their exponent range, so scores above m cost no
+                // precision until the sums near overflow.  The tile's row sum
+                // tells: past RAISE (or not a number) the row's m is raised to
+                // its max, O and l are rescaled, and the tile is done again
+                // from the scores still in registers.  (The commit behind
+                // s_full covers P V of tile g - 1, so O_i is stable.)  With a
+                // max for every tile / without: 12960 x 38880 x 40 heads 6.30
+                // / 6.20 ms, 12 heads 1.84 / 1.81 ms; at hd 64, where the
+                // other tile's exponentials hide the max, 0.494 / 0.555 ms.
+                // (P V issued from the first two or three quarters while the
+                // softmax computes the rest: 1.94 to 2.01 ms at 12 heads.)
+                bool fix = fresh;
+                float2 rs;
+                for (int pass = 0;; ++pass) {
+                    if (__any_sync(0xffffffffu, fix)) {
+                        const float m_new = fmaxf(m, row_max(s) * sl2);
+                        const float alpha = fix && !fresh ? ex2_approx(m - m_new) : 1.0f;
+                        if (fix) m = m_new;
+                        if (!fresh) {
+                            l *= alpha;
+                            scale_o(alpha);
+                        }
+                    }
+                    rs0 = rs1 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int qt = 0; qt < 4; ++qt) exp_quarter(s, qt, sl2, m, tP, rs0, rs1);
+                    rs = __fadd2_rn(rs0, rs1);
+                    fix = !(rs.x + rs.y <= A::RAISE);
+                    if (pass > 0 || !__any_sync(0xffffffffu, fix)) break;
+                }
+                l += rs.x + rs.y;
+                tc_fence_before();
+                mbar_arrive(&p_full[wg]);
+                return true;
             }
+            const float m_new = row_max(s) * sl2;
+            if (fresh) m = m_new;
+            const bool grow = !fresh && m_new > m + A::LAZY;
+            const float alpha = grow ? ex2_approx(m - m_new) : 1.0f;
+            if (grow) m = m_new;
+            // P_i buffer free and O_i stable once P V of the previous tile is done
+            if (g >= 1) {
+                ok = mbar_wait(&pv_done[wg], (g - 1) & 1, err, ERR_WAIT_SOFTMAX);
+                __syncwarp();
+                if (!__all_sync(0xffffffffu, ok)) return false;
+                tc_fence_after();
+            }
+            if (__any_sync(0xffffffffu, grow)) scale_o(alpha);
             // The two warps of each SM sub-partition (quadrant q of WG 0 and
             // of WG 1) take turns on the exponential phase, which is bound
             // by the sub-partition's MUFU: WG 0 does tile g, then WG 1 tile
@@ -463,39 +548,16 @@ __global__ void __launch_bounds__(352, 1)
             // overlap the other's loads, max and MMA waits.  The hand-off is
             // per quadrant, so a slower sub-partition does not hold up the
             // others.
-            // (hd 128: the turns cost more than they save -- the exponential
-            // phase is a smaller share of a key tile's work; 7.27 -> 7.16 ms
-            // at the 14B shape, 1.91 -> 1.85 ms at the 1.3B shape)
-            if constexpr (A::SEP_P) {
-                if (wg == 1 || g > 0) {
-                    ok = mbar_wait(&turn[4 * wg + q], (wg == 1 ? g : g - 1) & 1, err, ERR_WAIT_SOFTMAX);
-                    __syncwarp();
-                    if (!__all_sync(0xffffffffu, ok)) return false;
-                }
+            // (hd 128 takes no turns: its exponential phase is a smaller share of
+            // a key tile's work)
+            if (wg == 1 || g > 0) {
+                ok = mbar_wait(&turn[4 * wg + q], (wg == 1 ? g : g - 1) & 1, err, ERR_WAIT_SOFTMAX);
+                __syncwarp();
+                if (!__all_sync(0xffffffffu, ok)) return false;
             }
-            // probabilities p = 2^(s * sl2 - m), packed bf16 pairs + row sum,
-            // stored to TMEM in four 32-key quarters
-            const float2 sc2 = make_float2(sl2, sl2), nm2 = make_float2(-m, -m);
-            float2 rs0 = make_float2(0.f, 0.f), rs1 = make_float2(0.f, 0.f);
+            // probabilities and row sum in four 32-key quarters
 #pragma unroll
-            for (int qt = 0; qt < 4; ++qt) {
-                uint32_t w[16];
-#pragma unroll
-                for (int k = 0; k < 16; k += 2) {
-                    const int c = 32 * qt + 2 * k;
-                    const float2 a = __ffma2_rn(make_float2(s[c], s[c + 1]), sc2, nm2);
-                    const float2 b = __ffma2_rn(make_float2(s[c + 2], s[c + 3]), sc2, nm2);
-                    const float2 pa = make_float2(ex2_approx(a.x), ex2_approx(a.y));
-                    const float2 pb = make_float2(ex2_approx(b.x), ex2_approx(b.y));
-                    rs0 = __fadd2_rn(rs0, pa);
-                    rs1 = __fadd2_rn(rs1, pb);
-                    __nv_bfloat162 h0 = __floats2bfloat162_rn(pa.x, pa.y);
-                    __nv_bfloat162 h1 = __floats2bfloat162_rn(pb.x, pb.y);
-                    w[k] = *reinterpret_cast<uint32_t *>(&h0);
-                    w[k + 1] = *reinterpret_cast<uint32_t *>(&h1);
-                }
-                tmem_st16u_sync(tP + 16 * qt, w);
-            }
+            for (int qt = 0; qt < 4; ++qt) exp_quarter(s, qt, sl2, m, tP, rs0, rs1);
             const float2 rs = __fadd2_rn(rs0, rs1);
             l = l * alpha + (rs.x + rs.y);
             tc_fence_before();
@@ -511,27 +573,59 @@ __global__ void __launch_bounds__(352, 1)
             __syncwarp();
             if (!__all_sync(0xffffffffu, ok)) return false;
             tc_fence_after();
+            // through this warp's 4 KB of shared memory: a thread's own row
+            // stores to global memory touch 32 lines per instruction and took
+            // 5 us of a 256-query piece at hd 128
             const int h = u / sp.n_qblk;
-            const int row = (u % sp.n_qblk) * (A::QT * A::BQ) + r_tile;
+            const int row0 = (u % sp.n_qblk) * (A::QT * A::BQ) + wg * A::BQ + q * 32;   // this warp's first row
+            uint8_t *so = smem + A::OFF_O + warp * 4096 + lane * 128;
+            const int sw = lane & 7;
+            auto buffer_free = [&]() {                 // the last block's store has read it
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+            };
             if (!head_part && !cut_front) {
                 const float inv = 1.0f / l;
 #pragma unroll 1
-                for (int c = 0; c < HD / 16; ++c) {
-                    float t[16];
-                    tmem_ld16_sync(tO + 16 * c, t);
+                for (int c = 0; c < HD / 64; ++c) {
+                    float t[64];
+                    tmem_ld64_sync(tO + 64 * c, t);
+                    buffer_free();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) t[i] *= inv;
-                    if (row < Lq) store16<bf16>(o + (size_t)row * d + h * HD + 16 * c, t);
+                    for (int k = 0; k < 8; ++k) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            __nv_bfloat162 b2 = __floats2bfloat162_rn(t[8 * k + 2 * e] * inv, t[8 * k + 2 * e + 1] * inv);
+                            w[e] = *reinterpret_cast<uint32_t *>(&b2);
+                        }
+                        *reinterpret_cast<uint4 *>(so + ((k ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0 && row0 < Lq) {      // rows past Lq are clipped
+                        tma_store_2d(&tmO, smem + A::OFF_O + warp * 4096, h * HD + 64 * c, row0);
+                        bulk_commit();
+                    }
                 }
             } else {
                 const int slot = WAVE ? 2 * cta + (p - sp.W)                       // remainder piece 0 / 1
                                       : (head_part ? 2 * (cta + 1) : 2 * cta + 1);   // boundary c + 1 head / c tail
-                float *wo = ws_o + ((size_t)slot * (A::QT * A::BQ) + r_tile) * HD;
 #pragma unroll 1
-                for (int c = 0; c < HD / 16; ++c) {
-                    float t[16];
-                    tmem_ld16_sync(tO + 16 * c, t);
-                    store16<float>(wo + 16 * c, t);
+                for (int c = 0; c < HD / 32; ++c) {
+                    float t[32];
+                    tmem_ld32_sync(tO + 32 * c, t);
+                    buffer_free();
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        *reinterpret_cast<float4 *>(so + ((k ^ sw) << 4)) =
+                            make_float4(t[4 * k], t[4 * k + 1], t[4 * k + 2], t[4 * k + 3]);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        bulk_store(ws_o + partial_block(slot, warp, c, HD), smem + A::OFF_O + warp * 4096, 4096);
+                        bulk_commit();
+                    }
                 }
                 ws_ml[(size_t)slot * (A::QT * A::BQ) + r_tile] = make_float2(m, l);
             }
@@ -556,6 +650,9 @@ __global__ void __launch_bounds__(352, 1)
             ok = end_piece(cur.g, cur.u, piece_of(cur), cur.k != nkt - 1, cut_front, m, l);
             next(cur);
         }
+        // every store of this warp has completed before the CTA exits
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        __syncwarp();
     }
     tc_fence_before();
     __syncthreads();
@@ -566,84 +663,117 @@ __global__ void __launch_bounds__(352, 1)
 }
 
 // Merges the partials of the units cut between CTAs (see AttnSplit): m =
-// max_p m_p, O = sum_p O_p 2^(m_p - m) / sum_p l_p 2^(m_p - m).  Contiguous
+// max_p m_p, O = sum of O_p 2^(m_p - m) / sum of l_p 2^(m_p - m).  Contiguous
 // order: grid.x = CTA boundaries, two partials (head and tail) of the unit
 // the boundary cuts.  Waves: grid.x = remaining units, the partials of the
-// CTAs whose pieces touch it, in CTA order (up to G / R of them).  grid.y
-// picks 32 of the head's columns, grid.z 64 of the unit's 256 query rows;
-// one thread per row.
-constexpr int COMBINE_ROWS = 64, COMBINE_COLS = 32;
+// CTAs whose pieces touch it, in CTA order (at most G / units + 2).  grid.y
+// picks 32 of the head's columns, grid.z 32 of the unit's 256 query rows, 16
+// per warp.  The threads first find the partials' slots (one each: the share
+// bounds take 64-bit divisions, which one thread walking them alone spent
+// longer on than on the data), then every warp the weights 2^(m_p - m) / l of
+// its rows, and then it runs over the partials with four in flight, a lane
+// taking 4 columns of every fourth row (a load reads 512 contiguous bytes).
+// 19 partials of 8 units, hd 128: 35 us with one thread per row.
+constexpr int COMBINE_ROWS = 32, COMBINE_COLS = 32;
 template <int HD, bool WAVE>
-__global__ void __launch_bounds__(COMBINE_ROWS)
-    attn_combine_kernel(bf16 *__restrict__ o, const int Lq, const int d, const AttnSplit sp,
+__global__ void __launch_bounds__(64)
+    attn_combine_kernel(bf16 *__restrict__ o, const int Lq, const int d, const AttnSplit sp, const int max_part,
                         const float *__restrict__ ws_o, const float2 *__restrict__ ws_ml,
                         const uint8_t *__restrict__ skip_flag) {
     pdl_wait();
     if (skip_flag != nullptr && *skip_flag == XC_DEC_SKIP) return;
-    int u, c_lo, c_hi;
-    long long ub = 0;
+    extern __shared__ int comb_smem[];                 // slots [max_part], weights [2 warps][max_part][16]
+    int *slots = comb_smem;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *wgt = reinterpret_cast<float *>(comb_smem + max_part) + warp * max_part * 16;
+    int u, n;
     if constexpr (WAVE) {
         const int rr = blockIdx.x;                     // remaining unit
-        ub = (long long)rr * sp.n_kt;
-        const long long ue = ub + sp.n_kt;
-        c_lo = (int)(ub * sp.G / sp.T2);               // begin2(c_lo) <= ub
-        while (c_lo + 1 < sp.G && sp.begin2(c_lo + 1) <= ub) ++c_lo;
-        c_hi = c_lo;                                   // last CTA whose piece touches the unit
-        while (c_hi + 1 < sp.G && sp.begin2(c_hi + 1) < ue) ++c_hi;
-        if (c_hi == c_lo) return;                      // one CTA ran the whole unit and wrote it
+        const long long ub = (long long)rr * sp.n_kt, ue = ub + sp.n_kt;
         u = sp.W * sp.G + rr;
+        int c0 = (int)(ub * sp.G / sp.T2);             // begin2(c0) <= ub: the first CTA that can touch the unit
+        if (sp.begin2(c0 + 1) <= ub) ++c0;
+        // CTAs c0 .. c0 + n - 1 touch it; slot 2 c (its first piece) or 2 c + 1
+        n = 0;
+        for (int base = c0; base < sp.G; base += 64) {
+            const int c = base + threadIdx.x;
+            const long long b = sp.begin2(c), e = sp.begin2(c + 1);
+            const bool touch = c < sp.G && b < ue;
+            const int k = c - c0;
+            if (touch && k < max_part) slots[k] = e > b ? 2 * c + (b >= ub ? 0 : 1) : -1;
+            const int hit = __syncthreads_count(touch);
+            n += hit;
+            if (hit < 64) break;
+        }
+        n = min(n, max_part);
+        if (n == 1) return;                            // one CTA ran the whole unit and wrote it
     } else {
         const int b = blockIdx.x + 1;                  // boundary between CTAs b-1 and b
         const long long it = sp.begin(b);
         if (it % sp.n_kt == 0) return;                 // the boundary falls between units
         u = (int)(it / sp.n_kt);
-        c_lo = b - 1;
-        c_hi = b;
+        n = 2;
+        if (threadIdx.x < 2) slots[threadIdx.x] = 2 * b + threadIdx.x;         // head, tail
+        __syncthreads();
     }
     const int h = u / sp.n_qblk;
-    const int r = blockIdx.z * COMBINE_ROWS + threadIdx.x;     // row of the unit
-    const int k0 = blockIdx.y * COMBINE_COLS;
-    const int row = (u % sp.n_qblk) * 256 + r;
-    if (row >= Lq) return;
-    // slot of CTA c's partial of this unit
-    auto slot = [&](int c) {
-        if constexpr (WAVE) return 2 * c + (sp.begin2(c) >= ub ? 0 : 1);
-        else return c == c_lo ? 2 * c_hi : 2 * c_hi + 1;
-    };
-    auto has = [&](int c) {
-        if constexpr (WAVE) return sp.begin2(c + 1) > sp.begin2(c);
-        else return true;
-    };
-    float mm = -INFINITY;
-    for (int c = c_lo; c <= c_hi; ++c)
-        if (has(c)) mm = fmaxf(mm, ws_ml[(size_t)slot(c) * 256 + r].x);
-    float den = 0.0f;
-    float acc[COMBINE_COLS];
+    const int r16 = blockIdx.z * COMBINE_ROWS + warp * 16;                     // the warp's first row of the unit
+    const int row0 = (u % sp.n_qblk) * 256 + r16;
+    if (row0 >= Lq) return;
+    {   // weights: lane -> row lane % 16, every second partial
+        const float2 *ml = ws_ml + r16 + (lane & 15);
+        float m = -INFINITY, l = 0.0f;
+#pragma unroll 4
+        for (int p = lane >> 4; p < n; p += 2)
+            if (slots[p] >= 0) m = fmaxf(m, ml[(size_t)slots[p] * 256].x);
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+#pragma unroll 4
+        for (int p = lane >> 4; p < n; p += 2) {
+            float w = 0.0f;
+            if (slots[p] >= 0) {
+                const float2 t = ml[(size_t)slots[p] * 256];
+                w = exp2f(t.x - m);
+                l = fmaf(t.y, w, l);
+            }
+            wgt[p * 16 + (lane & 15)] = w;
+        }
+        l += __shfl_xor_sync(0xffffffffu, l, 16);
+        const float inv = 1.0f / l;
+        for (int p = lane >> 4; p < n; p += 2) wgt[p * 16 + (lane & 15)] *= inv;
+        __syncwarp();
+    }
+    constexpr int NR = 4;                              // rows of a lane: lr, lr + 4, ...
+    const int lr = lane >> 3, ch = lane & 7;
+    const int w8 = r16 >> 5, b16 = r16 & 31;           // softmax warp that wrote the rows, row of its block
+    float4 acc[NR];
 #pragma unroll
-    for (int i = 0; i < COMBINE_COLS; ++i) acc[i] = 0.0f;
-#pragma unroll 2
-    for (int c = c_lo; c <= c_hi; ++c) {
-        if (!has(c)) continue;
-        const int sl = slot(c);
-        const float2 ml = ws_ml[(size_t)sl * 256 + r];
-        const float w = exp2f(ml.x - mm);
-        den += ml.y * w;
-        const float *src = ws_o + ((size_t)sl * 256 + r) * HD + k0;
+    for (int i = 0; i < NR; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int p = 0; p < n; ++p) {
+        const int sl = slots[p];
+        if (sl < 0) continue;
+        const float4 *src = reinterpret_cast<const float4 *>(ws_o + partial_block(sl, w8, blockIdx.y, HD));
 #pragma unroll
-        for (int j = 0; j < COMBINE_COLS; j += 16) {
-            float x[16];
-            load16<float>(src + j, x);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) acc[j + i] = fmaf(x[i], w, acc[j + i]);
+        for (int i = 0; i < NR; ++i) {
+            const float4 x = src[(b16 + lr + 4 * i) * 8 + ch];                 // chunk ch ^ (row & 7) of its row
+            const float w = wgt[p * 16 + lr + 4 * i];
+            acc[i].x = fmaf(x.x, w, acc[i].x);
+            acc[i].y = fmaf(x.y, w, acc[i].y);
+            acc[i].z = fmaf(x.z, w, acc[i].z);
+            acc[i].w = fmaf(x.w, w, acc[i].w);
         }
     }
-    const float inv = 1.0f / den;
 #pragma unroll
-    for (int j = 0; j < COMBINE_COLS; j += 16) {
-        float y[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) y[i] = acc[j + i] * inv;
-        store16<bf16>(o + (size_t)row * d + h * HD + k0 + j, y);
+    for (int i = 0; i < NR; ++i) {
+        const int r = lr + 4 * i;
+        if (row0 + r >= Lq) break;
+        __nv_bfloat162 lo = __floats2bfloat162_rn(acc[i].x, acc[i].y);
+        __nv_bfloat162 hi = __floats2bfloat162_rn(acc[i].z, acc[i].w);
+        uint2 pk;
+        pk.x = *reinterpret_cast<uint32_t *>(&lo);
+        pk.y = *reinterpret_cast<uint32_t *>(&hi);
+        *reinterpret_cast<uint2 *>(o + (size_t)(row0 + r) * d + h * HD + blockIdx.y * COMBINE_COLS +
+                                   4 * (ch ^ ((b16 + r) & 7))) = pk;
     }
 }
 
@@ -665,9 +795,10 @@ size_t attn_workspace_bytes(int head_dim) {
 }
 
 template <int HD, bool WAVE>
-static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, bf16 *o,
-                                int Lq, int n_keys, int d, const AttnSplit &sp, bool split, int n_combine, void *ws,
-                                const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {
+static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                                const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int d, const AttnSplit &sp,
+                                int n_combine, void *ws, const uint8_t *skip, int *err, int *n_launched,
+                                cudaStream_t st) {
     using A = AttnTile<HD>;
     static bool attr_set = false;
     if (!attr_set) {
@@ -677,63 +808,93 @@ static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, co
         attr_set = true;
     }
     const int n_sm = sm_count();
-    float *ws_o = split ? reinterpret_cast<float *>(ws) : nullptr;
-    float2 *ws_ml = split ? reinterpret_cast<float2 *>(ws_o + 2 * ((size_t)n_sm + 1) * 256 * HD) : nullptr;
+    float *ws_o = n_combine > 0 ? reinterpret_cast<float *>(ws) : nullptr;
+    float2 *ws_ml = n_combine > 0 ? reinterpret_cast<float2 *>(ws_o + 2 * ((size_t)n_sm + 1) * 256 * HD) : nullptr;
     cudaError_t e = launch_pdl(attn_tc_kernel<HD, WAVE>, dim3(sp.G), dim3(A::THREADS), A::SMEM_BYTES, st, tq, tk,
-                               tv, o, Lq, n_keys, d, sp, ws_o, ws_ml, skip, err);
+                               tv, to, Lq, n_keys, sp, ws_o, ws_ml, skip, err);
     if (e != cudaSuccess) return e;
     if (n_launched) *n_launched = 1;
-    if (split && n_combine > 0) {
-        e = launch_pdl(attn_combine_kernel<HD, WAVE>, dim3(n_combine, HD / COMBINE_COLS, 256 / COMBINE_ROWS),
-                       dim3(COMBINE_ROWS), 0, st, o, Lq, d, sp,
+    if (n_combine > 0) {
+        const int max_part = WAVE ? std::min(sp.G, sp.G / n_combine + 2) : 2;
+        e = launch_pdl(attn_combine_kernel<HD, WAVE>, dim3(n_combine, HD / COMBINE_COLS, 256 / COMBINE_ROWS), dim3(64),
+                       (size_t)max_part * 33 * sizeof(float), st, o, Lq, d, sp, max_part,
                        static_cast<const float *>(ws_o), static_cast<const float2 *>(ws_ml), skip);
         if (n_launched) *n_launched = 2;
     }
     return e;
 }
 
-// Work order (see AttnSplit): waves when there are many of them (W >= 8)
-// and the K / V of all heads exceed L2 -- measured at the 14B shape (40
-// heads x 20 MB of K / V, W = 13): 40.7 -> 1.2 GB of DRAM traffic per launch
-// at the same attention time, the GPU's power then allowing a higher clock
-// under its cap (1500 -> 1965 MHz, 0.766 -> 0.801 chunks/s); at the 1.3B
-// shape (W = 4) the waves were 28 % slower per launch, the contiguous order
-// stays.
+// Work order (see AttnSplit).  Cutting units balances the SMs at the price of
+// partials and their merge, CUT key tiles' time or so.
+//  * Whole units in waves where the longest CTA has at most CUT key tiles
+//    more than an even share (cross-attention to a few hundred condition
+//    tokens: 12960 x 300 x 12 heads of 128 60.8 us cut, 37.1 whole), and
+//    without a workspace.
+//  * Fewer units than SMs: every unit is split over the same number of CTAs,
+//    so that no CTA touches two units; more than half as many units as SMs,
+//    over all SMs.  One CTA per unit before: 840 x 2520 x 4 heads of 64 26.6
+//    -> 16.2 us, 1000 x 10000 x 2 heads of 128 118 -> 28.
+//  * Waves with the remaining units split when there are many waves (W >= 8)
+//    and the K / V of all heads exceed L2 -- measured at the 14B shape (40
+//    heads x 20 MB of K / V, W = 13): 40.7 -> 1.2 GB of DRAM traffic per
+//    launch at the same attention time, the GPU's power then allowing a
+//    higher clock under its cap (1500 -> 1965 MHz, 0.766 -> 0.801 chunks/s).
+//  * Else contiguous shares; at the 1.3B shape (W = 4) the waves were 4 %
+//    slower per launch.
 template <int HD>
-static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, bf16 *o,
-                               int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes,
-                               const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {
+static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                               const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws,
+                               size_t ws_bytes, const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {
     using A = AttnTile<HD>;
+    constexpr int CUT = 5;
     AttnSplit sp;
     sp.n_kt = (n_keys + A::BKV - 1) / A::BKV;
     sp.n_qblk = (Lq + A::QT * A::BQ - 1) / (A::QT * A::BQ);
     const int n_units = sp.n_qblk * n_heads;
-    sp.T = (long long)n_units * sp.n_kt;
     const int n_sm = sm_count();
-    const bool split = n_units > n_sm && ws != nullptr && ws_bytes >= attn_workspace_bytes(HD);
-    sp.G = split ? n_sm : n_units;
+    const bool can_cut = ws != nullptr && ws_bytes >= attn_workspace_bytes(HD);
+    sp.T = (long long)n_units * sp.n_kt;
+    sp.T2 = 0;
+    sp.G = n_units < n_sm ? n_units : n_sm;
     sp.W = n_units / sp.G;
-    const int n_rem = n_units - sp.W * sp.G;
-    sp.T2 = (long long)n_rem * sp.n_kt;
+    sp.R = n_units - sp.W * sp.G;
+    const long long longest = (long long)(sp.W + (sp.R > 0 ? 1 : 0)) * sp.n_kt;
+    if (!can_cut || (longest - CUT) * n_sm <= sp.T)
+        return launch_attn_<HD, true>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 0, ws, skip, err, n_launched, st);
+    if (n_units < n_sm) {
+        // CTAs per unit: a key tile takes a CTA about 1.2 us and a partial the
+        // merge about 0.4, so some sqrt(3 n_kt) of them are best (300 x 30000
+        // x 1 head of 128: 76 / 59 / 40 per unit 66 / 53 / 43 us; 474 x 8116 x
+        // 2 heads of 64: 32 / 16 / 11 30 / 21.8 / 21.3)
+        int per = 1;
+        while (per * per < 3 * sp.n_kt) ++per;
+        per = std::min(per, std::min(n_sm / n_units, (sp.n_kt + 1) / 2));
+        sp.G = per >= 2 ? n_units * per : n_sm;
+        sp.W = sp.R = 0;
+        sp.T2 = sp.T;
+        return launch_attn_<HD, true>(tq, tk, tv, to, o, Lq, n_keys, d, sp, n_units, ws, skip, err, n_launched, st);
+    }
     const double kv_bytes = 2.0 * n_keys * (double)d * sizeof(bf16);
-    const bool wave = split && sp.W >= 8 && kv_bytes > 128.0 * 1024 * 1024;
-    if (wave)
-        return launch_attn_<HD, true>(tq, tk, tv, o, Lq, n_keys, d, sp, split, n_rem, ws, skip, err, n_launched, st);
-    return launch_attn_<HD, false>(tq, tk, tv, o, Lq, n_keys, d, sp, split, sp.G - 1, ws, skip, err, n_launched,
-                                   st);
+    if (sp.W >= 8 && kv_bytes > 128.0 * 1024 * 1024) {
+        const int n_rem = sp.R;
+        sp.T2 = (long long)n_rem * sp.n_kt;
+        sp.R = 0;
+        return launch_attn_<HD, true>(tq, tk, tv, to, o, Lq, n_keys, d, sp, n_rem, ws, skip, err, n_launched, st);
+    }
+    return launch_attn_<HD, false>(tq, tk, tv, to, o, Lq, n_keys, d, sp, sp.G - 1, ws, skip, err, n_launched, st);
 }
 
-// q [Lq][d], k / v maps over [>= n_keys][d] (box 128 rows), o [Lq][d]; hd in {64, 128}.
-// ws: attn_workspace_bytes(hd) bytes enable the balanced split over the SMs
-// when there are more units than SMs (nullptr: one CTA per unit).
+// q [Lq][d], k / v maps over [>= n_keys][d] (boxes of 128 rows), o [Lq][d] and
+// its map (boxes of 32 rows); hd in {64, 128}.  ws: attn_workspace_bytes(hd)
+// bytes let units be cut between CTAs (nullptr: whole units only).
 cudaError_t attn_tc(int head_dim, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
-                    bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes,
+                    const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes,
                     const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {
     if (n_keys < 1 || Lq < 1) return cudaErrorInvalidValue;
     if (head_dim == 64)
-        return launch_attn<64>(tq, tk, tv, o, Lq, n_keys, n_heads, d, ws, ws_bytes, skip, err, n_launched, st);
+        return launch_attn<64>(tq, tk, tv, to, o, Lq, n_keys, n_heads, d, ws, ws_bytes, skip, err, n_launched, st);
     if (head_dim == 128)
-        return launch_attn<128>(tq, tk, tv, o, Lq, n_keys, n_heads, d, ws, ws_bytes, skip, err, n_launched, st);
+        return launch_attn<128>(tq, tk, tv, to, o, Lq, n_keys, n_heads, d, ws, ws_bytes, skip, err, n_launched, st);
     return cudaErrorInvalidValue;
 }
 

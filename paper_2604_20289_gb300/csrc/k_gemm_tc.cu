@@ -102,18 +102,6 @@ struct EpiMaps {
 // bf16 block (the layout TMA reads and writes with CU_TENSOR_MAP_SWIZZLE_64B).
 __device__ __forceinline__ uint32_t sw64(int r, int k) { return (uint32_t)(r * 64 + ((k ^ ((r >> 1) & 3)) << 4)); }
 
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap *tm, const void *src, int x, int y) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                 ::"l"(reinterpret_cast<uint64_t>(tm)), "r"(smem_u32(src)), "r"(x), "r"(y)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() {
-    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // (a, b) += (x, y), (a, b) = (x a + r, y b + s): packed fp32 pairs
 __device__ __forceinline__ void add2(float &a, float &b, float x, float y) {
     const float2 t = __fadd2_rn(make_float2(a, b), make_float2(x, y));

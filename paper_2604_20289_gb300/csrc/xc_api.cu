@@ -216,7 +216,7 @@ struct xc_ctx {
     cudaStream_t cap_st;                       // capture stream (the caller's may be the legacy default)
 
     // tensor maps (bf16); output tile width of each GEMM
-    CUtensorMap tm_h, tm_o, tm_u, tm_q;
+    CUtensorMap tm_h, tm_o, tm_u, tm_q, tm_ao;   // tm_ao: o as the attention writes it
     int bn_qkv, bn_o, bn_f1, bn_f2, bn_caq;
     std::vector<WeightMaps> tm_wqkv, tm_wo, tm_w1, tm_w2;
     std::vector<CUtensorMap> tm_rk, tm_rv;
@@ -699,7 +699,7 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
         if constexpr (sizeof(T) == 2) {
             int n_attn = 1;
             LAUNCH(XC_K_ATTN, b, n_attn,
-                   attn_tc(hd, ctx->tm_q, ctx->tm_rk[b], ctx->tm_rv[b], reinterpret_cast<bf16 *>(ob), L, n_keys,
+                   attn_tc(hd, ctx->tm_q, ctx->tm_rk[b], ctx->tm_rv[b], ctx->tm_ao, reinterpret_cast<bf16 *>(ob), L, n_keys,
                            ctx->H, d, ctx->attn_ws, ctx->attn_ws_bytes, flag, ctx->d_err, &n_attn, st));
         } else {
             const float *Kr = reinterpret_cast<const float *>(ctx->ring_k) + (size_t)b * ctx->Wkv * Ld;
@@ -738,7 +738,7 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
                        gemm_tc(EPI_BIAS, ctx->bn_caq, ctx->tm_h, ctx->tm_caq[b], ep, d, flag, ctx->d_err, st));
                 int n_x = 1;
                 LAUNCH(XC_K_XATTN, b, n_x,
-                       attn_tc(hd, ctx->tm_q, ctx->tm_ck[b], ctx->tm_cv[b], reinterpret_cast<bf16 *>(ob), L,
+                       attn_tc(hd, ctx->tm_q, ctx->tm_ck[b], ctx->tm_cv[b], ctx->tm_ao, reinterpret_cast<bf16 *>(ob), L,
                                ctx->n_ctx, ctx->H, d, ctx->attn_ws, ctx->attn_ws_bytes, flag, ctx->d_err, &n_x, st));
             } else {
                 const float *W = reinterpret_cast<const float *>(ctx->ca_q_wt) + (size_t)b * d * d;
@@ -1131,6 +1131,7 @@ xc_status xc_init(const xc_model_cfg *cfg, const xc_weights *w, void *cuda_strea
             ctx->bn_f2 = gemm_tc_bn(EPI_RESID_CACHE, L, d, F);
             tmap(ctx, &ctx->tm_h, ctx->hbuf, L, d, 128);
             tmap(ctx, &ctx->tm_o, ctx->o, L, d, 128);
+            tmap(ctx, &ctx->tm_ao, ctx->o, L, d, 32);
             tmap(ctx, &ctx->tm_u, ctx->u, L, F, 128);
             tmap(ctx, &ctx->tm_q, ctx->q, L, d, 128);
             ctx->tm_wqkv.resize(B);
@@ -1655,11 +1656,11 @@ xc_status xc_op_attention(int dtype, int Lq, int n_keys, int n_heads, int head_d
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (dtype == XC_BF16) {
         if (head_dim != 64 && head_dim != 128) OP_FAIL(XC_EINVAL, "xc_op_attention: bf16 head_dim 64 or 128");
-        CUtensorMap tq, tk, tv;
+        CUtensorMap tq, tk, tv, to;
         if (!make_tmap_bf16(&tq, q, Lq, d, 128) || !make_tmap_bf16(&tk, k, n_keys, d, 128) ||
-            !make_tmap_bf16(&tv, v, n_keys, d, 128))
+            !make_tmap_bf16(&tv, v, n_keys, d, 128) || !make_tmap_bf16(&to, o, Lq, d, 32))
             OP_FAIL(XC_EINVAL, "xc_op_attention: tensor map");
-        OP_CK(attn_tc(head_dim, tq, tk, tv, reinterpret_cast<bf16 *>(o), Lq, n_keys, n_heads, d, workspace,
+        OP_CK(attn_tc(head_dim, tq, tk, tv, to, reinterpret_cast<bf16 *>(o), Lq, n_keys, n_heads, d, workspace,
                       workspace_bytes, nullptr, op_err_word(), nullptr, st));
     } else if (dtype == XC_F32) {
         OP_CK(attn_simt(head_dim, reinterpret_cast<const float *>(q), reinterpret_cast<const float *>(k),

@@ -98,8 +98,8 @@ inline bool make_weight_maps(WeightMaps *m, const void *base, uint64_t N, uint64
 int gemm_tc_bn(int epi, int M, int N, int K);
 cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                     const uint8_t *skip, int *err, cudaStream_t st);
-cudaError_t attn_tc(int head_dim, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, bf16 *o,
-                    int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes, const uint8_t *skip, int *err,
+cudaError_t attn_tc(int head_dim, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                    const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes, const uint8_t *skip, int *err,
                     int *n_launched, cudaStream_t st);
 size_t attn_workspace_bytes(int head_dim);
 cudaError_t gemm_simt(int epi, const EpiParams &ep, const float *A, const float *Wt, int K, const uint8_t *skip,
