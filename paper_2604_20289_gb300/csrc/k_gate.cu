@@ -16,8 +16,10 @@
 // the longer each row's contiguous run), the row blocks split each camera's
 // tokens so that the grid fills the SMs (up to four CTAs per SM), and the R
 // row blocks of one (camera, slice) form a thread-block cluster.  A CTA
-// streams its rows of its slice once (16-byte streaming loads, batches of 8
-// rows in flight per thread) into column sums, and takes every R-th row of
+// streams its rows of its slice once (16-byte loads, batches of 8 rows in
+// flight per thread; kept in L2, since the reuse path or the block's LN reads
+// the input next: gate + reuse at 12960 x 1536 40.1 us with evict-first loads,
+// 37.4 without) into column sums, and takes every R-th row of
 // the camera's spatial sample in its slice.  Two folds follow, each in a
 // fixed order (deterministic; the only waits are one cluster barrier, which
 // every CTA of the cluster reaches, and no spin-wait):
@@ -128,13 +130,13 @@ __device__ __forceinline__ void slice_colsums(const T *x, size_t ctok0, int d, i
     for (; i + GATE_UNROLL <= n; i += GATE_UNROLL) {
         uint4 u[GATE_UNROLL];
 #pragma unroll
-        for (int k = 0; k < GATE_UNROLL; ++k) u[k] = __ldcs(reinterpret_cast<const uint4 *>(p + k * stride));
+        for (int k = 0; k < GATE_UNROLL; ++k) u[k] = *reinterpret_cast<const uint4 *>(p + k * stride);
         p += GATE_UNROLL * stride;
 #pragma unroll
         for (int k = 0; k < GATE_UNROLL; ++k) add_pairs<T>(acc2, u[k]);
     }
     for (; i < n; ++i) {
-        add_pairs<T>(acc2, __ldcs(reinterpret_cast<const uint4 *>(p)));
+        add_pairs<T>(acc2, *reinterpret_cast<const uint4 *>(p));
         p += stride;
     }
 #pragma unroll
@@ -193,6 +195,20 @@ __global__ void __launch_bounds__(GATE_THREADS, GATE_CTAS_PER_SM) gate_kernel(co
     const float *phi_prev = g.phi + (size_t)active * n_all;
     float *phi_next = g.phi + (size_t)(active ^ 1) * n_all;
     cg::cluster_group cluster = cg::this_cluster();
+    // What thread 0 of the last CTA needs at the end, loaded now (nothing
+    // writes it before the decision): the chains of dependent loads there were
+    // on the launch's critical path.
+    GateCell cell{};
+    float act_cur = 0.0f, act_prev = 0.0f;
+    bool replay_skip = false;
+    if (tid < g.A) {
+        act_cur = g.action_dev != nullptr ? g.action_dev[tid] : g.action[tid];
+        act_prev = g.phi_act[active * 8 + tid];
+    }
+    if (tid == 0) {
+        cell = *g.cell;
+        if (g.replay_dev != nullptr) replay_skip = *g.replay_dev != 0;
+    }
 
     // 1. column sums of rows [rb0, rb1) of camera c, columns [col0, col0 + cw),
     //    into rank 0's shared memory -- unless the previous block was skipped
@@ -305,25 +321,25 @@ __global__ void __launch_bounds__(GATE_THREADS, GATE_CTAS_PER_SM) gate_kernel(co
         }
         __syncthreads();
     }
+    if (warp != 0) return;
+    // condition entry: lanes < A hold the action's components (A <= 8), added in lane order
+    float da = 0.0f, na = 0.0f, nb = 0.0f;
+    for (int i = 0; i < g.A; ++i) {
+        const float a = __shfl_sync(0xffffffffu, act_cur, i), b = __shfl_sync(0xffffffffu, act_prev, i);
+        da = fmaf(a, b, da);
+        na = fmaf(a, a, na);
+        nb = fmaf(b, b, nb);
+    }
+    if (lane < g.A) g.phi_act[(active ^ 1) * 8 + lane] = act_cur;
     if (tid != 0) return;
     *g.ticket = 0u;
 
     // All sums and metrics are fp32 (relative error ~1e-7, far inside the
     // 1e-3 band around a threshold): FP64 arithmetic, square roots and divides
     // are slow on this part; only the EMA state stays fp64.
-    float da = 0.0f, na = 0.0f, nb = 0.0f;
-    for (int i = 0; i < g.A; ++i) {
-        const float a = g.action_dev != nullptr ? g.action_dev[i] : g.action[i];
-        const float b = g.phi_act[active * 8 + i];
-        da = fmaf(a, b, da);
-        na = fmaf(a, a, na);
-        nb = fmaf(b, b, nb);
-        g.phi_act[(active ^ 1) * 8 + i] = a;
-    }
     const float cos_a = cos_rule_f(da, na, nb);
     const double s_min = (double)fminf(cos_min, cos_a);
 
-    GateCell cell = *g.cell;
     uint8_t dec;
     bool flip;
     if (g.mode == 1 && cell.valid) {
@@ -332,7 +348,7 @@ __global__ void __launch_bounds__(GATE_THREADS, GATE_CTAS_PER_SM) gate_kernel(co
         bool skip = (s_min >= tau) && (dmax < g.tau_dev);
         if (g.max_skips > 0 && cell.stale >= g.max_skips) skip = false;
         if (g.replay_dev != nullptr)
-            skip = *g.replay_dev != 0;
+            skip = replay_skip;
         else if (g.replay >= 0)
             skip = g.replay != 0;
         cell.ema = cell.has_hist ? (double)g.alpha * s_min + (1.0 - (double)g.alpha) * cell.ema : s_min;
