@@ -1,6 +1,8 @@
 // Bandwidth-bound and small kernels of the chunk step: patch embedding,
 // adaLN-Zero LayerNorm modulation, the reuse path (Eq. 4), the conditioning
 // GEMVs, the output head, the Euler update and weight layout conversion.
+#include <algorithm>
+
 #include "xc_kernels.cuh"
 #include "xc_ptx.cuh"
 
@@ -46,9 +48,16 @@ constexpr int PE_COLS = 128, PE_WARPS = 8, PE_CHUNK = 64;
 template <typename T>
 __global__ void __launch_bounds__(PE_WARPS * 32)
     patch_embed_kernel(const float *__restrict__ z, const float *__restrict__ w, const float *__restrict__ b,
-                       T *__restrict__ out, int L, int d, int rows_per_cta) {
+                       T *__restrict__ out, int L, int d, int rows_per_cta, uint8_t *__restrict__ flags,
+                       float *__restrict__ metrics, int B) {
     pdl_wait();
     pdl_release();
+    // the pass's decisions start as "forced", its metrics (3 per block) as NaN
+    if (flags != nullptr && blockIdx.x == 0 && blockIdx.y == 0)
+        for (int i = threadIdx.x; i < 3 * B; i += blockDim.x) {
+            metrics[i] = __int_as_float(-1);
+            if (i < B) flags[i] = 0;
+        }
     __shared__ __align__(16) float zs[2][PE_CHUNK * 16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = blockIdx.x * PE_COLS + 4 * lane;
@@ -114,7 +123,8 @@ __global__ void __launch_bounds__(PE_WARPS * 32)
 }
 
 template <typename T>
-cudaError_t patch_embed(const float *z, const float *w, const float *b, T *out, int L, int C, int d, cudaStream_t st) {
+cudaError_t patch_embed(const float *z, const float *w, const float *b, T *out, int L, int C, int d, uint8_t *flags,
+                        float *metrics, int B, cudaStream_t st) {
     if (C != 16 || d % 16 != 0) return cudaErrorInvalidValue;
     const int n_sm = n_sm_elem();
     const int n_cb = (d + PE_COLS - 1) / PE_COLS;
@@ -122,10 +132,12 @@ cudaError_t patch_embed(const float *z, const float *w, const float *b, T *out, 
     const int rows = ((L + n_rb - 1) / n_rb + PE_CHUNK - 1) / PE_CHUNK * PE_CHUNK;
     n_rb = (L + rows - 1) / rows;
     return launch_pdl(patch_embed_kernel<T>, dim3(n_cb, n_rb < 1 ? 1 : n_rb), dim3(PE_WARPS * 32), 0, st, z, w, b,
-                      out, L, d, rows);
+                      out, L, d, rows, flags, metrics, B);
 }
-template cudaError_t patch_embed<float>(const float *, const float *, const float *, float *, int, int, int, cudaStream_t);
-template cudaError_t patch_embed<bf16>(const float *, const float *, const float *, bf16 *, int, int, int, cudaStream_t);
+template cudaError_t patch_embed<float>(const float *, const float *, const float *, float *, int, int, int, uint8_t *,
+                                        float *, int, cudaStream_t);
+template cudaError_t patch_embed<bf16>(const float *, const float *, const float *, bf16 *, int, int, int, uint8_t *,
+                                       float *, int, cudaStream_t);
 
 // ------------------------------------------------------------- row stats
 // A row is walked in 16-element runs; lane l owns runs l, l + 32, ...  Each
@@ -156,76 +168,9 @@ __device__ __forceinline__ Moments warp_moments(Moments a) {
     }
     return a;
 }
-// Moments of the first n_valid of the NCH runs a lane holds in registers.
-template <int NCH>
-__device__ __forceinline__ Moments lane_moments(const float (&v)[NCH][16], int n_valid) {
-    float s = 0.0f;
-#pragma unroll
-    for (int k = 0; k < NCH; ++k)
-        if (k < n_valid) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) s += v[k][i];
-        }
-    Moments m = {16.0f * n_valid, 0.0f, 0.0f};
-    if (n_valid == 0) return m;
-    m.mean = s / m.n;
-#pragma unroll
-    for (int k = 0; k < NCH; ++k)
-        if (k < n_valid) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float t = v[k][i] - m.mean;
-                m.m2 = fmaf(t, t, m.m2);
-            }
-        }
-    return m;
-}
-
 // ----------------------------------------------------------------- ln_mod
-// One warp per row, the row held in registers (d <= 512 * NCH):
 // h = round(LN(x) * (1 + scale) + shift).
-template <typename T, int NCH>
-__global__ void __launch_bounds__(256)
-    ln_mod_kernel(const T *__restrict__ x, const float *__restrict__ shift, const float *__restrict__ scale,
-                  T *__restrict__ out, int M, int d, float eps, const uint8_t *__restrict__ skip_flag) {
-    pdl_wait();
-    pdl_release();
-    if (skip_flag != nullptr && *skip_flag == XC_DEC_SKIP) return;
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= M) return;
-    const T *xr = x + (size_t)row * d;
-    const int runs = d / 16;
-    const int mine = runs > lane ? (runs - lane + 31) / 32 : 0;
-    float v[NCH][16];
-#pragma unroll
-    for (int k = 0; k < NCH; ++k)
-        if (k < mine) load16<T>(xr + 16 * (lane + 32 * k), v[k]);
-    // the modulation vectors do not depend on the moments: fetch them while
-    // the row reduction runs (one chunk ahead for wide rows)
-    float sc[16], sh[16];
-    if (mine > 0) {
-        load16<float>(scale + 16 * lane, sc);
-        load16<float>(shift + 16 * lane, sh);
-    }
-    const Moments mo = warp_moments(lane_moments<NCH>(v, mine));
-    const float rstd = rsqrtf(mo.m2 / (float)d + eps);
-    T *orow = out + (size_t)row * d;
-#pragma unroll
-    for (int k = 0; k < NCH; ++k) {
-        if (k < mine) {
-            const int c = 16 * (lane + 32 * k);
-            if (k > 0) {
-                load16<float>(scale + c, sc);
-                load16<float>(shift + c, sh);
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[k][i] = (v[k][i] - mo.mean) * rstd * (1.0f + sc[i]) + sh[i];
-            store16<T>(orow + c, v[k]);
-        }
-    }
-}
-
+//
 // d <= 512 (one 16-element run per lane): persistent warps walk rows
 // row, row + n_warps, ... with the next row's load in flight while the
 // current one is reduced; the modulation vectors stay in registers.
@@ -277,11 +222,15 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// d > 512: one CTA of LN_CTA threads per row.  The row is loaded once into
-// registers as packed 16-byte vectors (KMAX per thread, all loads in flight),
-// the mean and then the squared deviations are reduced over the CTA (warp
-// butterflies, then the warps in order), and the modulated row is written
-// back; many rows per SM are in flight at once.
+// d > 512: one CTA of LN_CTA threads per ROWS (1 or 2) rows.  The rows are
+// loaded once into registers as packed 16-byte vectors (KMAX per thread and
+// row, all loads in flight), the means and then the squared deviations are
+// reduced over the CTA (warp butterflies, then the warps in order), and the
+// modulated rows are written back; many rows per SM are in flight at once.
+// Bound by DRAM, beside it by L1: the modulation vectors are twice the bytes
+// of a bf16 row, so two rows share one read of them (12960 x 5120 bf16: one
+// row per CTA 50.0 us, two 45.9 = 5.8 TB/s; 256 threads 62, 64 threads 52;
+// persistent CTAs with the vectors in registers 79).
 constexpr int LN_CTA = 128;
 
 template <typename T>
@@ -316,19 +265,25 @@ __device__ __forceinline__ uint4 pack16B(const float (&f)[16 / sizeof(T)]) {
     }
 }
 
-// Sum over the CTA in a fixed order (deterministic).
-__device__ __forceinline__ float cta_sum(float v, float *red) {
+// Sums over the CTA in a fixed order (deterministic).
+template <int ROWS>
+__device__ __forceinline__ void cta_sum(float (&v)[ROWS], float (*red)[ROWS]) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[r] += __shfl_xor_sync(0xffffffffu, v[r], o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][r] = v[r];
+    }
     __syncthreads();
-    float s = red[0];
 #pragma unroll
-    for (int w = 1; w < LN_CTA / 32; ++w) s += red[w];
-    return s;
+    for (int r = 0; r < ROWS; ++r) {
+        v[r] = red[0][r];
+#pragma unroll
+        for (int w = 1; w < LN_CTA / 32; ++w) v[r] += red[w][r];
+    }
 }
 
-template <typename T, int KMAX>
+template <typename T, int KMAX, int ROWS>
 __global__ void __launch_bounds__(LN_CTA)
     ln_mod_cta_kernel(const T *__restrict__ x, const float *__restrict__ shift, const float *__restrict__ scale,
                       T *__restrict__ out, int M, int d, float eps, const uint8_t *__restrict__ skip_flag) {
@@ -336,44 +291,55 @@ __global__ void __launch_bounds__(LN_CTA)
     pdl_release();
     if (skip_flag != nullptr && *skip_flag == XC_DEC_SKIP) return;
     constexpr int VEC = 16 / sizeof(T);
-    __shared__ float red[2][LN_CTA / 32];
-    const int row = blockIdx.x, tid = threadIdx.x;
-    if (row >= M) return;
+    __shared__ float red[2][LN_CTA / 32][ROWS];
+    const int row = ROWS * blockIdx.x, tid = threadIdx.x;
+    const int n_rows = min(ROWS, M - row);             // the last CTA may have one
     const int nch = d / VEC;
     const uint4 *xr = reinterpret_cast<const uint4 *>(x + (size_t)row * d);
-    uint4 raw[KMAX];
+    uint4 raw[ROWS][KMAX];
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        const int c = tid + k * LN_CTA;
-        raw[k] = c < nch ? xr[c] : make_uint4(0u, 0u, 0u, 0u);
-    }
-    float s = 0.0f;
+    for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        float f[VEC];
-        unpack16B<T>(raw[k], f);
+        for (int k = 0; k < KMAX; ++k) {
+            const int c = tid + k * LN_CTA;
+            raw[r][k] = c < nch && r < n_rows ? xr[(size_t)r * nch + c] : make_uint4(0u, 0u, 0u, 0u);
+        }
+    float mean[ROWS], rstd[ROWS];
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) s += f[i];
-    }
-    const float mean = cta_sum(s, red[0]) / (float)d;
-    float m2 = 0.0f;
+    for (int r = 0; r < ROWS; ++r) {
+        mean[r] = 0.0f;
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        if (tid + k * LN_CTA < nch) {
+        for (int k = 0; k < KMAX; ++k) {
             float f[VEC];
-            unpack16B<T>(raw[k], f);
+            unpack16B<T>(raw[r][k], f);
 #pragma unroll
-            for (int i = 0; i < VEC; ++i) m2 = fmaf(f[i] - mean, f[i] - mean, m2);
+            for (int i = 0; i < VEC; ++i) mean[r] += f[i];
         }
     }
-    const float rstd = rsqrtf(cta_sum(m2, red[1]) / (float)d + eps);
+    cta_sum<ROWS>(mean, red[0]);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        mean[r] /= (float)d;
+        rstd[r] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < KMAX; ++k) {
+            if (tid + k * LN_CTA < nch) {
+                float f[VEC];
+                unpack16B<T>(raw[r][k], f);
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) rstd[r] = fmaf(f[i] - mean[r], f[i] - mean[r], rstd[r]);
+            }
+        }
+    }
+    cta_sum<ROWS>(rstd, red[1]);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) rstd[r] = rsqrtf(rstd[r] / (float)d + eps);
     uint4 *orow = reinterpret_cast<uint4 *>(out + (size_t)row * d);
 #pragma unroll
     for (int k = 0; k < KMAX; ++k) {
         const int c = tid + k * LN_CTA;
         if (c < nch) {
-            float f[VEC], sc[VEC], sh[VEC];
-            unpack16B<T>(raw[k], f);
+            float sc[VEC], sh[VEC];
 #pragma unroll
             for (int i = 0; i < VEC; i += 4) {
                 const float4 a = *reinterpret_cast<const float4 *>(scale + (size_t)c * VEC + i);
@@ -382,8 +348,14 @@ __global__ void __launch_bounds__(LN_CTA)
                 sh[i] = b.x; sh[i + 1] = b.y; sh[i + 2] = b.z; sh[i + 3] = b.w;
             }
 #pragma unroll
-            for (int i = 0; i < VEC; ++i) f[i] = (f[i] - mean) * rstd * (1.0f + sc[i]) + sh[i];
-            orow[c] = pack16B<T>(f);
+            for (int r = 0; r < ROWS; ++r) {
+                if (r >= n_rows) break;
+                float f[VEC];
+                unpack16B<T>(raw[r][k], f);
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) f[i] = (f[i] - mean[r]) * rstd[r] * (1.0f + sc[i]) + sh[i];
+                orow[(size_t)r * nch + c] = pack16B<T>(f);
+            }
         }
     }
 }
@@ -391,14 +363,14 @@ __global__ void __launch_bounds__(LN_CTA)
 template <typename T, int KMAX>
 static cudaError_t ln_mod_cta(const T *x, const float *shift, const float *scale, T *out, int M, int d, float eps,
                               const uint8_t *skip, cudaStream_t st) {
-    return launch_pdl(ln_mod_cta_kernel<T, KMAX>, dim3(M), dim3(LN_CTA), 0, st, x, shift, scale, out, M, d, eps,
-                      skip);
-}
-
-template <typename T, int NCH>
-static cudaError_t ln_mod_n(const T *x, const float *shift, const float *scale, T *out, int M, int d, float eps,
-                            const uint8_t *skip, cudaStream_t st) {
-    return launch_pdl(ln_mod_kernel<T, NCH>, dim3((M + 7) / 8), dim3(256), 0, st, x, shift, scale, out, M, d, eps, skip);
+    // two rows per CTA for 16-bit rows (fp32 rows are as long as the vectors:
+    // 2000 x 5120 15.1 us with one, 16.6 with two) while every SM still gets
+    // several CTAs (200 x 4368: 3.4 us with one, 3.6 with two)
+    if constexpr (sizeof(T) == 2)
+        if (M >= 4 * n_sm_elem())
+            return launch_pdl(ln_mod_cta_kernel<T, KMAX, 2>, dim3((M + 1) / 2), dim3(LN_CTA), 0, st, x, shift, scale, out,
+                              M, d, eps, skip);
+    return launch_pdl(ln_mod_cta_kernel<T, KMAX, 1>, dim3(M), dim3(LN_CTA), 0, st, x, shift, scale, out, M, d, eps, skip);
 }
 
 template <typename T>
@@ -409,7 +381,7 @@ cudaError_t ln_mod(const T *x, const float *shift, const float *scale, T *out, i
         const int want = (M + 7) / 8, cap = 2 * n_sm_elem();
         return launch_pdl(ln_mod_row_kernel<T>, dim3(want < cap ? want : cap), dim3(256), 0, st, x, shift, scale, out, M, d, eps, skip);
     }
-    // one CTA per row: 16-byte vectors per thread
+    // 16-byte vectors per thread
     const int per = (d / (16 / (int)sizeof(T)) + LN_CTA - 1) / LN_CTA;
     if (per <= 2) return ln_mod_cta<T, 2>(x, shift, scale, out, M, d, eps, skip, st);
     if (per <= 4) return ln_mod_cta<T, 4>(x, shift, scale, out, M, d, eps, skip, st);
@@ -417,10 +389,7 @@ cudaError_t ln_mod(const T *x, const float *shift, const float *scale, T *out, i
     if (per <= 6) return ln_mod_cta<T, 6>(x, shift, scale, out, M, d, eps, skip, st);
     if (per <= 8) return ln_mod_cta<T, 8>(x, shift, scale, out, M, d, eps, skip, st);
     if (per <= 12) return ln_mod_cta<T, 12>(x, shift, scale, out, M, d, eps, skip, st);
-    switch ((d + 511) / 512) {
-        case 9: case 10: case 11: case 12: return ln_mod_n<T, 12>(x, shift, scale, out, M, d, eps, skip, st);
-        default: return cudaErrorInvalidValue;
-    }
+    return cudaErrorInvalidValue;
 }
 template cudaError_t ln_mod<float>(const float *, const float *, const float *, float *, int, int, float,
                                    const uint8_t *, cudaStream_t);
@@ -522,11 +491,50 @@ cudaError_t euler_update(float *x, const float *v, float ds, long n, cudaStream_
     return launch_pdl(euler_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, x, v, ds, n);
 }
 
+// ------------------------------------------------------------ RoPE table
+// (cos, sin) of one chunk, double precision.  Axes (camera, frame, h, w) own
+// hd/16, 3hd/16, hd/8, hd/8 consecutive pairs; pair j of an axis with D = 2 *
+// pairs dims rotates at theta^(-2j/D).  Axis a has npos[a] positions (frame:
+// the chunk's frames, absolute frame = frame0 + p); entry base_a + j * npos[a]
+// + p holds (cos, sin)(pos * freq).  With axis / off set, also every pair's
+// axis and the entry of its position 0.
+// One warp per CTA does 32 entries: double precision runs at two FMA per clock
+// and SM, so several warps in one CTA wait for each other.
+__device__ __forceinline__ void rope_entry(const RopeArgs &r, int e) {
+    const int hd = r.hd;
+    const int pairs[4] = {hd / 16, 3 * hd / 16, hd / 8, hd / 8};
+    const int np[4] = {r.npos.x, r.npos.y, r.npos.z, r.npos.w};
+    // this entry's axis first, so that a warp whose entries span several axes
+    // runs the double-precision functions once
+    int base = 0, pair0 = 0, j = 0, n_pairs = 0, pos = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const int span = pairs[a] * np[a];
+        if (r.axis != nullptr && e >= pair0 && e < pair0 + pairs[a]) {
+            r.axis[e] = a;
+            r.off[e] = base + (e - pair0) * np[a];
+        }
+        if (e >= base && e < base + span) {
+            j = (e - base) / np[a];
+            pos = (e - base) % np[a] + (a == 1 ? r.frame0 : 0);
+            n_pairs = pairs[a];
+        }
+        base += span;
+        pair0 += pairs[a];
+    }
+    if (n_pairs == 0) return;
+    const double ang = (double)pos * pow(r.theta, -2.0 * j / (2.0 * n_pairs));
+    double sn, cs;
+    sincos(ang, &sn, &cs);
+    r.out[e] = make_float2((float)cs, (float)sn);
+}
+
 // ----------------------------------------------------------- conditioning
 constexpr int GEMV_WARPS = 16;
 
 // Fused conditioning (a2), three launches per pass:
-//   stage 1: ht = SiLU(W_t1 temb + b_t1), ha = SiLU(W_a1 a + b_a1)
+//   stage 1: ht = SiLU(W_t1 temb + b_t1), ha = SiLU(W_a1 a + b_a1), and in
+//            CTAs of its own the chunk's RoPE table
 //   stage 2: e  = (W_t2 ht + b_t2) + (W_a2 ha + b_a2)
 //   stage 3: mods[b] = W_m SiLU(e) + b_m + table_b (every block b),
 //            hmod    = W_h SiLU(e) + b_h + table_head
@@ -564,6 +572,10 @@ __global__ void __launch_bounds__(GEMV_WARPS * 32) cond_kernel(const CondArgs c)
     int j = 0, n_out = d;
     float acc = 0.0f;
     if constexpr (STAGE == 1) {
+        if ((int)blockIdx.x >= 2 * nb_d) {
+            if (warp == 0) rope_entry(c.rope, (blockIdx.x - 2 * nb_d) * 32 + lane);
+            return;
+        }
         const bool tpath = (int)blockIdx.x < nb_d;
         j = (tpath ? blockIdx.x : blockIdx.x - nb_d) * 32 + lane;
         const int n_in = tpath ? c.tf : c.A;
@@ -631,7 +643,7 @@ cudaError_t conditioning(const CondArgs &c, cudaStream_t st) {
     if (c.A < 1 || c.A > 8 || c.tf < 2 || c.tf > COND_TEMB_MAX || (size_t)2 * d * sizeof(float) > 48 * 1024)
         return cudaErrorInvalidValue;
     const int in1 = c.tf > c.A ? c.tf : c.A;
-    cudaError_t e = launch_pdl(cond_kernel<1>, dim3(2 * nb_d), dim3(GEMV_WARPS * 32), in1 * sizeof(float), st, c);
+    cudaError_t e = launch_pdl(cond_kernel<1>, dim3(2 * nb_d + (c.rope.n + 31) / 32), dim3(GEMV_WARPS * 32), in1 * sizeof(float), st, c);
     if (e != cudaSuccess) return e;
     e = launch_pdl(cond_kernel<2>, dim3(nb_d), dim3(GEMV_WARPS * 32), 2 * d * sizeof(float), st, c);
     if (e != cudaSuccess) return e;
@@ -639,35 +651,16 @@ cudaError_t conditioning(const CondArgs &c, cudaStream_t st) {
                       d * sizeof(float), st, c);
 }
 
-// RoPE (cos, sin) table of one chunk, double precision.  Axes (camera, frame,
-// h, w) own hd/16, 3hd/16, hd/8, hd/8 consecutive pairs; pair j of an axis
-// with D = 2 * pairs dims rotates at theta^(-2j/D).  Axis a has npos[a]
-// positions (frame: the chunk's frames, absolute frame = frame0 + p); entry
-// base_a + j * npos[a] + p holds (cos, sin)(pos * freq).
-__global__ void rope_table_kernel(int hd, double theta, int frame0, int4 npos, float2 *__restrict__ out, int n) {
+// RoPE table and pair layout of one chunk as a launch of its own (operator
+// path; the chunk step's conditioning writes its table).
+__global__ void __launch_bounds__(32) rope_table_kernel(const RopeArgs r) {
     pdl_wait();
     pdl_release();
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int pairs[4] = {hd / 16, 3 * hd / 16, hd / 8, hd / 8};
-    const int np[4] = {npos.x, npos.y, npos.z, npos.w};
-    int base = 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int span = pairs[a] * np[a];
-        if (e < base + span) {
-            const int j = (e - base) / np[a];
-            const int p = (e - base) % np[a];
-            const double freq = pow(theta, -2.0 * j / (2.0 * pairs[a]));
-            const double ang = (double)(p + (a == 1 ? frame0 : 0)) * freq;
-            out[e] = make_float2((float)cos(ang), (float)sin(ang));
-            return;
-        }
-        base += span;
-    }
+    rope_entry(r, blockIdx.x * 32 + threadIdx.x);
 }
-cudaError_t rope_table(int hd, double theta, int frame0, int4 npos, float2 *out, int n, cudaStream_t st) {
-    return launch_pdl(rope_table_kernel, dim3((n + 127) / 128), dim3(128), 0, st, hd, theta, frame0, npos, out, n);
+cudaError_t rope_table(const RopeArgs &r, cudaStream_t st) {
+    const int n = std::max(r.n, r.hd / 2);
+    return launch_pdl(rope_table_kernel, dim3((n + 31) / 32), dim3(32), 0, st, r);
 }
 
 // ------------------------------------------------------------------- head

@@ -561,13 +561,15 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
         ca.head_w = ctx->head_w; ca.head_b = ctx->head_b; ca.head_tab = ctx->head_tab;
         ca.ht = ctx->ht; ca.ha = ctx->ha; ca.e = ctx->e; ca.mods = ctx->mods; ca.hmod = ctx->hmod;
         ca.act_out = ctx->act_dev;
+        // RoPE table of this chunk (absolute frames n*F .. n*F + F - 1)
+        ca.rope.hd = hd;
+        ca.rope.theta = (double)ctx->cfg.rope_theta;
+        ca.rope.frame0 = n * ctx->cfg.frames;
+        ca.rope.npos = make_int4(ctx->V, ctx->cfg.frames, ctx->rope_h, ctx->rope_w);
+        ca.rope.out = ctx->rope_cs;
+        ca.rope.n = ctx->rope_n;
         LAUNCH(XC_K_COND, -1, 3, conditioning(ca, st));
     }
-    // RoPE table of this chunk (absolute frames n*F .. n*F + F - 1)
-    LAUNCH(XC_K_EMBED, -1, 1,
-           rope_table(hd, (double)ctx->cfg.rope_theta, n * ctx->cfg.frames,
-                      make_int4(ctx->V, ctx->cfg.frames, ctx->rope_h, ctx->rope_w), ctx->rope_cs,
-                      ctx->rope_n, st));
 
     // Everything below takes from the host only what PassSig holds, so it is
     // captured into a CUDA graph and replayed for passes with the same
@@ -580,9 +582,8 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
     // only needs every block's K/V: the last block stops after its K/V
     // projection and the head is not run.
     const bool kv_tail_off = kv && !want_v && ctx->trace == nullptr;
-    LAUNCH(XC_K_EMBED, -1, 1, patch_embed<T>(lat_dev, ctx->pe_w, ctx->pe_b, X[0], L, ctx->C, d, st));
-    CK(cudaMemsetAsync(ctx->flags, 0, B, st));
-    CK(cudaMemsetAsync(ctx->s_cos, 0xFF, 3 * B * sizeof(float), st));   // NaN
+    LAUNCH(XC_K_EMBED, -1, 1, patch_embed<T>(lat_dev, ctx->pe_w, ctx->pe_b, X[0], L, ctx->C, d, ctx->flags,
+                                                ctx->s_cos, B, st));
 
     const bool gating = p.enabled != 0 && !kv;
     const bool eval_mode = eval_pass(ctx, p, t);
@@ -1605,10 +1606,17 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
         OP_CK(cudaMalloc(&off, cap_pairs * sizeof(int)));
         OP_CK(cudaMalloc(&cs, cap_entries * sizeof(float2)));
     }
-    OP_CK(cudaMemcpyAsync(axis, ax.data(), ax.size() * sizeof(int), cudaMemcpyHostToDevice, st0));
-    OP_CK(cudaMemcpyAsync(off, of.data(), of.size() * sizeof(int), cudaMemcpyHostToDevice, st0));
-    OP_CK(rope_table(head_dim, (double)rope_theta, chunk * frames, make_int4(n_cams, frames, gh, gw), cs, n_entries,
-                     st0));
+    // table and pair layout written on the device: no host copies in the call
+    RopeArgs ra{};
+    ra.hd = head_dim;
+    ra.theta = (double)rope_theta;
+    ra.frame0 = chunk * frames;
+    ra.npos = make_int4(n_cams, frames, gh, gw);
+    ra.out = cs;
+    ra.n = n_entries;
+    ra.axis = axis;
+    ra.off = off;
+    OP_CK(rope_table(ra, st0));
     const int npc = frames * gh * gw, M = n_cams * npc;
     EpiParams ep;
     memset(&ep, 0, sizeof ep);

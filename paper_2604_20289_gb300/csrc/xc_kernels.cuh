@@ -107,7 +107,8 @@ cudaError_t gemm_simt(int epi, const EpiParams &ep, const float *A, const float 
 cudaError_t attn_simt(int head_dim, const float *q, const float *k, const float *v, float *o, int Lq, int n_keys,
                       int H, const uint8_t *skip, cudaStream_t st);
 template <typename T>
-cudaError_t patch_embed(const float *z, const float *w, const float *b, T *out, int L, int C, int d, cudaStream_t st);
+cudaError_t patch_embed(const float *z, const float *w, const float *b, T *out, int L, int C, int d, uint8_t *flags,
+                        float *metrics, int B, cudaStream_t st);
 template <typename T>
 cudaError_t ln_mod(const T *x, const float *shift, const float *scale, T *out, int M, int d, float eps,
                    const uint8_t *skip, cudaStream_t st);
@@ -116,6 +117,15 @@ cudaError_t residual_reuse(const T *x, const T *r, T *out, long n, const uint8_t
 cudaError_t euler_update(float *x, const float *v, float ds, long n, cudaStream_t st);
 template <typename T>
 cudaError_t convert_f32(const float *in, T *out, long n, int n_sm, cudaStream_t st);
+// RoPE (cos, sin) table of a chunk: n entries to out; axis / off (or nullptr):
+// every pair's axis and first entry.
+struct RopeArgs {
+    int hd, frame0, n;
+    double theta;
+    int4 npos;
+    float2 *out;
+    int *axis, *off;
+};
 // Fused conditioning (three launches), see k_elem.cu.
 constexpr int COND_TEMB_MAX = 512;
 struct CondArgs {
@@ -126,13 +136,14 @@ struct CondArgs {
     const float *mod_w, *mod_b, *blk_mod, *head_w, *head_b, *head_tab;
     float *ht, *ha, *e, *mods, *hmod;
     float *act_out;               // device copy of the action (read by the gate kernels)
+    RopeArgs rope;
 };
 cudaError_t conditioning(const CondArgs &c, cudaStream_t st);
 template <typename T>
 cudaError_t head(const T *x, const float *hm, const float *w, const float *b, float *v, int L, int d, float eps,
                  cudaStream_t st);
 template <typename T> cudaError_t transpose_convert(const float *W, T *Wt, int K, int N, cudaStream_t st);
-cudaError_t rope_table(int hd, double theta, int frame0, int4 npos, float2 *out, int n, cudaStream_t st);
+cudaError_t rope_table(const RopeArgs &r, cudaStream_t st);
 // Test of the bounded waits: a one-thread kernel whose wait runs out (after
 // WAIT_NS) and records `code` in *err.
 cudaError_t expire_wait(int *err, int code, cudaStream_t st);
