@@ -1565,9 +1565,9 @@ xc_status xc_op_linear(int dtype, int epilogue, int M, int N, int K, const void 
     if (dtype == XC_BF16) {
         if (N % 256 != 0 || K % 64 != 0) OP_FAIL(XC_EINVAL, "xc_op_linear: bf16 needs N %% 256 == 0, K %% 64 == 0");
         CUtensorMap ta;
-        WeightMaps tb;
+        WeightMaps tb{};
         const int bn = gemm_tc_bn(epilogue, M, N, K);
-        if (!make_tmap_bf16(&ta, A, M, K, 128) || !make_weight_maps(&tb, Wt, N, K))
+        if (!make_tmap_bf16(&ta, A, M, K, 128) || !make_weight_maps(&tb, bn, Wt, N, K))
             OP_FAIL(XC_EINVAL, "xc_op_linear: tensor map (alignment?)");
         OP_CK(gemm_tc(epilogue, bn, ta, tb, ep, K, nullptr, op_err_word(), st));
     } else if (dtype == XC_F32) {
@@ -1637,9 +1637,9 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
     if (dtype == XC_BF16) {
         if ((3 * d) % 256 != 0 || d % 64 != 0) OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: bf16 needs 3d %% 256, d %% 64");
         CUtensorMap ta;
-        WeightMaps tb;
+        WeightMaps tb{};
         const int bn = gemm_tc_bn(EPI_QKV_ROPE, M, 3 * d, d);
-        if (!make_tmap_bf16(&ta, A, M, d, 128) || !make_weight_maps(&tb, Wt, 3 * (uint64_t)d, d))
+        if (!make_tmap_bf16(&ta, A, M, d, 128) || !make_weight_maps(&tb, bn, Wt, 3 * (uint64_t)d, d))
             OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: tensor map");
         OP_CK(gemm_tc(EPI_QKV_ROPE, bn, ta, tb, ep, d, nullptr, op_err_word(), st));
     } else if (dtype == XC_F32) {

@@ -92,8 +92,10 @@ bool make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t co
 struct WeightMaps {
     CUtensorMap box128, box64;
 };
-inline bool make_weight_maps(WeightMaps *m, const void *base, uint64_t N, uint64_t K) {
-    return make_tmap_bf16(&m->box128, base, N, K, 128) && make_tmap_bf16(&m->box64, base, N, K, 64);
+// The maps that tiling bn uses (0: all).
+inline bool make_weight_maps(WeightMaps *m, int bn, const void *base, uint64_t N, uint64_t K) {
+    if (bn != 64 && !make_tmap_bf16(&m->box128, base, N, K, 128)) return false;
+    return bn == 128 || make_tmap_bf16(&m->box64, base, N, K, 64);
 }
 int gemm_tc_bn(int epi, int M, int N, int K);
 cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,

@@ -155,6 +155,10 @@ def _ptr(t) -> int | None:
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            # the raw handle of torch.cuda.current_stream(), without the Stream
+            # object (0.2 against 3.1 us, a third of a small operator call)
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     return getattr(stream, "cuda_stream", stream)
 
