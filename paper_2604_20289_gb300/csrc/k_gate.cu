@@ -81,6 +81,47 @@ __device__ __forceinline__ void add_pairs(float2 (&acc)[16 / sizeof(T) / 2], con
     }
 }
 
+// N consecutive floats (16-byte vectors when al says that they are aligned).
+template <int N>
+__device__ __forceinline__ void load_vec(const float *p, float (&v)[N], bool al) {
+    if (al) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) {
+            const float4 t = *reinterpret_cast<const float4 *>(p + i);
+            v[i] = t.x; v[i + 1] = t.y; v[i + 2] = t.z; v[i + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = p[i];
+    }
+}
+template <int N>
+__device__ __forceinline__ void store_vec(float *p, const float (&v)[N], bool al) {
+    if (al) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) *reinterpret_cast<float4 *>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) p[i] = v[i];
+    }
+}
+// 16 bytes of an activation row.
+template <typename T>
+__device__ __forceinline__ void load_row(const T *p, float (&v)[16 / sizeof(T)]) {
+    const uint4 u = *reinterpret_cast<const uint4 *>(p);
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+    if constexpr (sizeof(T) == 2) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[2 * j] = __uint_as_float(w[j] << 16);
+            v[2 * j + 1] = __uint_as_float(w[j] & 0xFFFF0000u);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = __uint_as_float(w[j]);
+    }
+}
+
 // Sum (or, for part 3, max) of the 8 partials over the CTA in a fixed order:
 // butterfly within each warp, then warps in index order by thread 0.
 __device__ __forceinline__ void cta_fold8(float (&v)[GATE_PARTS], float (*wpart)[GATE_PARTS], int lane, int warp,
@@ -220,31 +261,43 @@ __global__ void __launch_bounds__(GATE_THREADS, GATE_CTAS_PER_SM) gate_kernel(co
                          cluster);
 
     float p[GATE_PARTS] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    // 2. sample rows r, r + R, ... of camera c in this slice
+    // 2. sample rows r, r + R, ... of camera c in this slice: cw / VEC threads
+    //    to a row, 16 bytes of x each (one element per thread and iteration
+    //    was a chain of two dependent loads eight times over at d 5120: 10 of
+    //    the gate's 41 us)
     {
-        const int n_mine = r < kfp ? (kfp - r + R - 1) / R : 0;
-        for (int it = tid; it < n_mine * cw; it += GATE_THREADS) {
-            const int i = r + (it / cw) * R, j = it % cw;
-            const int row = g.fp_rows[crow0 + i];
-            const size_t e = ((size_t)crow0 + i) * d + col0 + j;
-            float cur;
+        const int TPR = cw / VEC, RPAR = GATE_THREADS / TPR;
+        const int col = col0 + (tid % TPR) * VEC;
+        const bool al = (reinterpret_cast<uintptr_t>(g.phi) & 15) == 0;
+        for (int i = r + (tid / TPR) * R; i < kfp; i += RPAR * R) {
+            const size_t xe = (size_t)g.fp_rows[crow0 + i] * d + col;
+            const size_t e = ((size_t)crow0 + i) * d + col;
+            float cur[VEC], prev[VEC];
+            load_vec<VEC>(phi_prev + e, prev, al);
             if (chained) {
                 // chained input on the sampled rows: running fp32 sum of the last
                 // materialised rows and the pending residuals, rounded once
-                const float sum = g.csp_in[e] + to_f(reinterpret_cast<const T *>(g.rhat_prev)[(size_t)row * d + col0 + j]);
-                g.csp_out[e] = sum;
-                cur = round_to<T>(sum);
+                float res[VEC];
+                load_row<T>(reinterpret_cast<const T *>(g.rhat_prev) + xe, res);
+                load_vec<VEC>(g.csp_in + e, cur, true);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) cur[k] += res[k];
+                store_vec<VEC>(g.csp_out + e, cur, true);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) cur[k] = round_to<T>(cur[k]);
             } else {
-                cur = to_f(x[(size_t)row * d + col0 + j]);
-                if (g.chain) g.csp_out[e] = cur;
+                load_row<T>(x + xe, cur);
+                if (g.chain) store_vec<VEC>(g.csp_out + e, cur, true);
             }
-            const float prev = phi_prev[e];
-            phi_next[e] = cur;
-            p[0] = fmaf(cur, prev, p[0]);
-            p[1] = fmaf(cur, cur, p[1]);
-            p[2] = fmaf(prev, prev, p[2]);
-            p[3] = fmaxf(p[3], fabsf(cur - prev));
-            p[4] += fabsf(prev);
+            store_vec<VEC>(phi_next + e, cur, al);
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                p[0] = fmaf(cur[k], prev[k], p[0]);
+                p[1] = fmaf(cur[k], cur[k], p[1]);
+                p[2] = fmaf(prev[k], prev[k], p[2]);
+                p[3] = fmaxf(p[3], fabsf(cur[k] - prev[k]));
+                p[4] += fabsf(prev[k]);
+            }
         }
     }
 
