@@ -138,6 +138,10 @@ __device__ __forceinline__ void exp_quarter(const float (&s)[128], int qt, float
 //    partial slots 2 c and 2 c + 1), merged per remaining unit by
 //    attn_combine_kernel.  With fewer units than SMs W = 0: every unit is
 //    such a remaining one.
+//  * clusters (ORDER_CLUSTER): as waves with W = 0 and every unit cut evenly
+//    over the CTAs of one thread-block cluster, which leave their partials in
+//    their shared memory and merge them there -- no second launch and no
+//    partials through global memory.
 // Each role walks the CTA's key tiles with a cursor (TileCursor): tile
 // counter g, unit u and its key tile k; in the wave order also the piece
 // index p and the unit step du.
@@ -185,12 +189,16 @@ __device__ __forceinline__ void bulk_store(void *dst, const void *src, uint32_t 
                  : "memory");
 }
 
-template <int HD, bool WAVE>
+// Work orders of attn_tc_kernel (see AttnSplit).
+enum { ORDER_CONTIGUOUS = 0, ORDER_WAVE = 1, ORDER_CLUSTER = 2 };
+
+template <int HD, int ORDER>
 __global__ void __launch_bounds__(352, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const int Lq,
-                   const int n_keys, const AttnSplit sp, float *__restrict__ ws_o,
+                   const int n_keys, const AttnSplit sp, bf16 *__restrict__ o, const int d, float *__restrict__ ws_o,
                    float2 *__restrict__ ws_ml, const uint8_t *__restrict__ skip_flag, int *err) {
+    constexpr bool WAVE = ORDER != ORDER_CONTIGUOUS, CLUSTER = ORDER == ORDER_CLUSTER;
     pdl_wait();
     using A = AttnTile<HD>;
     if (skip_flag != nullptr && *skip_flag == XC_DEC_SKIP) return;
@@ -212,7 +220,8 @@ __global__ void __launch_bounds__(352, 1)
     uint64_t *pv_done = p_full + 2;            // [2] P_i V done (hd 64: every tile; hd 128: last of a piece)
     uint64_t *o_free = pv_done + 2;            // [2] O_i of piece p read out (phase p)
     uint64_t *turn = o_free + 2;               // [2][4] exponential-phase hand-off per (WG, quadrant)
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(turn + 8);
+    uint64_t *all_pv = turn + 8;               // clusters: every P V of the CTA done (its K / V ring is free)
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(all_pv + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkt = sp.n_kt;
@@ -269,6 +278,7 @@ __global__ void __launch_bounds__(352, 1)
     if (threadIdx.x == 0) {
         mbar_init(q_full, 1);
         mbar_init(q_empty, A::ISSUERS);
+        mbar_init(all_pv, 256);
         for (int s = 0; s < A::STAGES; ++s) {
             mbar_init(&k_full[s], 1);
             mbar_init(&k_empty[s], A::ISSUERS);   // freed by every MMA warp
@@ -573,6 +583,26 @@ __global__ void __launch_bounds__(352, 1)
             __syncwarp();
             if (!__all_sync(0xffffffffu, ok)) return false;
             tc_fence_after();
+            if constexpr (CLUSTER) {
+                // unnormalised O and (m, l) stay in shared memory, O in the K / V
+                // ring once both Q tiles' last P V has read it
+                mbar_arrive(all_pv);
+                const bool done = mbar_wait(all_pv, 0, err, ERR_WAIT_SOFTMAX);
+                __syncwarp();
+                if (!__all_sync(0xffffffffu, done)) return false;
+#pragma unroll 1
+                for (int c = 0; c < HD / 32; ++c) {
+                    float t[32];
+                    tmem_ld32_sync(tO + 32 * c, t);
+                    uint8_t *blk = sK + partial_block(0, warp, c, HD) * sizeof(float) + lane * 128;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        *reinterpret_cast<float4 *>(blk + ((k ^ (lane & 7)) << 4)) =
+                            make_float4(t[4 * k], t[4 * k + 1], t[4 * k + 2], t[4 * k + 3]);
+                }
+                reinterpret_cast<float2 *>(smem + A::OFF_O)[r_tile] = make_float2(m, l);
+                return true;
+            }
             // through this warp's 4 KB of shared memory: a thread's own row
             // stores to global memory touch 32 lines per instruction and took
             // 5 us of a 256-query piece at hd 128
@@ -656,6 +686,68 @@ __global__ void __launch_bounds__(352, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (CLUSTER) {
+        // The cluster's partials: a warp takes 16 rows x 32 columns at a time,
+        // first the weights 2^(m_p - m) / l of its rows, then the weighted sum,
+        // a lane 4 columns of every fourth row.
+        cluster_sync_all();
+        const int n_cta = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
+        if (warp < 8) {
+            const int u = c0.u, h = u / sp.n_qblk;
+            float *wgt = reinterpret_cast<float *>(smem + A::OFF_O + 4096) + warp * 256;      // [16 CTAs][16 rows]
+            const int lr = lane >> 3, ch = lane & 7;
+            for (int b = rank * 8 + warp; b < 16 * (HD / 32); b += 8 * n_cta) {
+                const int r16 = (b & 15) * 16, grp = b >> 4;
+                const int row0 = (u % sp.n_qblk) * (A::QT * A::BQ) + r16;
+                if (row0 >= Lq) continue;
+                const float2 *ml = reinterpret_cast<const float2 *>(smem + A::OFF_O) + r16 + (lane & 15);
+                float mm = -INFINITY, l = 0.0f;
+                for (int p = lane >> 4; p < n_cta; p += 2) mm = fmaxf(mm, ld_cluster2(map_to_cta(ml, p)).x);
+                mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, 16));
+                for (int p = lane >> 4; p < n_cta; p += 2) {
+                    const float2 t = ld_cluster2(map_to_cta(ml, p));
+                    const float w = exp2f(t.x - mm);
+                    l = fmaf(t.y, w, l);
+                    wgt[p * 16 + (lane & 15)] = w;
+                }
+                l += __shfl_xor_sync(0xffffffffu, l, 16);
+                const float inv = 1.0f / l;
+                for (int p = lane >> 4; p < n_cta; p += 2) wgt[p * 16 + (lane & 15)] *= inv;
+                __syncwarp();
+                const uint8_t *blk = sK + partial_block(0, r16 >> 5, grp, HD) * sizeof(float) + (r16 & 31) * 128 + ch * 16;
+                float4 acc[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+                for (int p = 0; p < n_cta; ++p) {
+                    const uint32_t src = map_to_cta(blk, p);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 x = ld_cluster4(src + (lr + 4 * i) * 128);
+                        const float w = wgt[p * 16 + lr + 4 * i];
+                        acc[i].x = fmaf(x.x, w, acc[i].x);
+                        acc[i].y = fmaf(x.y, w, acc[i].y);
+                        acc[i].z = fmaf(x.z, w, acc[i].z);
+                        acc[i].w = fmaf(x.w, w, acc[i].w);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = lr + 4 * i;
+                    if (row0 + r >= Lq) break;
+                    __nv_bfloat162 lo = __floats2bfloat162_rn(acc[i].x, acc[i].y);
+                    __nv_bfloat162 hi = __floats2bfloat162_rn(acc[i].z, acc[i].w);
+                    uint2 pk;
+                    pk.x = *reinterpret_cast<uint32_t *>(&lo);
+                    pk.y = *reinterpret_cast<uint32_t *>(&hi);
+                    *reinterpret_cast<uint2 *>(o + (size_t)(row0 + r) * d + h * HD + 32 * grp +
+                                               4 * (ch ^ (r & 7))) = pk;
+                }
+                __syncwarp();
+            }
+        }
+        cluster_sync_all();                            // no CTA leaves while another reads its partials
+    }
     if (warp == 9) {
         tc_fence_after();
         tmem_dealloc(tmem, A::TMEM_COLS);
@@ -794,24 +886,58 @@ size_t attn_workspace_bytes(int head_dim) {
     return slots * 256 * ((size_t)head_dim * sizeof(float) + sizeof(float2));
 }
 
-template <int HD, bool WAVE>
-static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
-                                const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int d, const AttnSplit &sp,
-                                int n_combine, void *ws, const uint8_t *skip, int *err, int *n_launched,
-                                cudaStream_t st) {
+template <int HD, int ORDER>
+static cudaError_t attn_attr() {
     using A = AttnTile<HD>;
     static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<HD, WAVE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             A::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
+    if (attr_set) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<HD, ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               A::SMEM_BYTES);
+    attr_set = e == cudaSuccess;
+    return e;
+}
+
+// Clusters of `size` attention CTAs (one per SM) that are resident at once.
+template <int HD>
+static int attn_clusters(int size) {
+    static int known[9];                               // 0: not asked yet
+    if (known[size] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(size * (sm_count() / size)));
+        cfg.blockDim = dim3(AttnTile<HD>::THREADS);
+        cfg.dynamicSmemBytes = AttnTile<HD>::SMEM_BYTES;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (attn_attr<HD, ORDER_CLUSTER>() != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<HD, ORDER_CLUSTER>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        known[size] = n > 0 ? n : -1;
     }
+    return known[size];
+}
+
+template <int HD, int ORDER>
+static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                                const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int d, const AttnSplit &sp,
+                                int cluster, int n_combine, void *ws, const uint8_t *skip, int *err, int *n_launched,
+                                cudaStream_t st) {
+    using A = AttnTile<HD>;
+    constexpr bool WAVE = ORDER != ORDER_CONTIGUOUS;
+    cudaError_t e = attn_attr<HD, ORDER>();
+    if (e != cudaSuccess) return e;
     const int n_sm = sm_count();
     float *ws_o = n_combine > 0 ? reinterpret_cast<float *>(ws) : nullptr;
     float2 *ws_ml = n_combine > 0 ? reinterpret_cast<float2 *>(ws_o + 2 * ((size_t)n_sm + 1) * 256 * HD) : nullptr;
-    cudaError_t e = launch_pdl(attn_tc_kernel<HD, WAVE>, dim3(sp.G), dim3(A::THREADS), A::SMEM_BYTES, st, tq, tk,
-                               tv, to, Lq, n_keys, sp, ws_o, ws_ml, skip, err);
+    e = launch_pdl_cluster(attn_tc_kernel<HD, ORDER>, (unsigned)cluster, dim3(sp.G), dim3(A::THREADS), A::SMEM_BYTES, st,
+                           tq, tk, tv, to, Lq, n_keys, sp, o, d, ws_o, ws_ml, skip, err);
     if (e != cudaSuccess) return e;
     if (n_launched) *n_launched = 1;
     if (n_combine > 0) {
@@ -833,7 +959,7 @@ static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, co
 //  * Fewer units than SMs: every unit is split over the same number of CTAs,
 //    so that no CTA touches two units; more than half as many units as SMs,
 //    over all SMs.  One CTA per unit before: 840 x 2520 x 4 heads of 64 26.6
-//    -> 16.2 us, 1000 x 10000 x 2 heads of 128 118 -> 28.
+//    -> 16.2 us (14.3 in clusters), 1000 x 10000 x 2 heads of 128 118 -> 28.
 //  * Waves with the remaining units split when there are many waves (W >= 8)
 //    and the K / V of all heads exceed L2 -- measured at the 14B shape (40
 //    heads x 20 MB of K / V, W = 13): 40.7 -> 1.2 GB of DRAM traffic per
@@ -860,8 +986,26 @@ static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, con
     sp.R = n_units - sp.W * sp.G;
     const long long longest = (long long)(sp.W + (sp.R > 0 ? 1 : 0)) * sp.n_kt;
     if (!can_cut || (longest - CUT) * n_sm <= sp.T)
-        return launch_attn_<HD, true>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 0, ws, skip, err, n_launched, st);
+        return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, 0, ws, skip, err, n_launched, st);
     if (n_units < n_sm) {
+        // One cluster of up to 8 CTAs per unit, as many as can all be resident
+        // at once, while a CTA has at most 8 key tiles: beyond, more CTAs per
+        // unit gain more than their merge through global memory costs (1000 x
+        // 10000 x 2 heads of 128: 26.7 us by 16, 27.4 in clusters of 8).  At
+        // hd 128, with twice the partials, clusters of 3 and 4 lost: 840 x
+        // 2520 by 10 heads 22.8 -> 23.8 us, 8 heads 19.9 -> 20.2, 6 heads
+        // (clusters of 6) 20.4 -> 19.5; at hd 64 by 10 heads 18.8 -> 18.4, 6
+        // heads 17.4 -> 14.6, 4 heads 16.4 -> 14.3.
+        constexpr int CL_MIN = HD == 64 ? 2 : 6;
+        int cl = std::min(8, std::min(n_sm / n_units, (sp.n_kt + 1) / 2));
+        while (cl >= CL_MIN && n_units > attn_clusters<HD>(cl)) --cl;
+        if (cl >= CL_MIN && sp.n_kt <= 8 * cl) {
+            sp.G = n_units * cl;
+            sp.W = sp.R = 0;
+            sp.T2 = sp.T;
+            return launch_attn_<HD, ORDER_CLUSTER>(tq, tk, tv, to, o, Lq, n_keys, d, sp, cl, 0, ws, skip, err,
+                                                   n_launched, st);
+        }
         // CTAs per unit: a key tile takes a CTA about 1.2 us and a partial the
         // merge about 0.4, so some sqrt(3 n_kt) of them are best (300 x 30000
         // x 1 head of 128: 76 / 59 / 40 per unit 66 / 53 / 43 us; 474 x 8116 x
@@ -872,16 +1016,16 @@ static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, con
         sp.G = per >= 2 ? n_units * per : n_sm;
         sp.W = sp.R = 0;
         sp.T2 = sp.T;
-        return launch_attn_<HD, true>(tq, tk, tv, to, o, Lq, n_keys, d, sp, n_units, ws, skip, err, n_launched, st);
+        return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, n_units, ws, skip, err, n_launched, st);
     }
     const double kv_bytes = 2.0 * n_keys * (double)d * sizeof(bf16);
     if (sp.W >= 8 && kv_bytes > 128.0 * 1024 * 1024) {
         const int n_rem = sp.R;
         sp.T2 = (long long)n_rem * sp.n_kt;
         sp.R = 0;
-        return launch_attn_<HD, true>(tq, tk, tv, to, o, Lq, n_keys, d, sp, n_rem, ws, skip, err, n_launched, st);
+        return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, n_rem, ws, skip, err, n_launched, st);
     }
-    return launch_attn_<HD, false>(tq, tk, tv, to, o, Lq, n_keys, d, sp, sp.G - 1, ws, skip, err, n_launched, st);
+    return launch_attn_<HD, ORDER_CONTIGUOUS>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, sp.G - 1, ws, skip, err, n_launched, st);
 }
 
 // q [Lq][d], k / v maps over [>= n_keys][d] (boxes of 128 rows), o [Lq][d] and

@@ -40,12 +40,14 @@ def check(q, k, v, H, hd, workspace):
     assert xb.op_device_error() == 0
 
 
-# (Lq, Lk, H, hd) on 152 SMs: 16 units split evenly; one unit split many ways;
+# (Lq, Lk, H, hd) on 152 SMs: 16 units in clusters; one unit in a cluster of 8;
 # 90 units over all SMs (shares touch two units); 2 units of 3 tiles; whole
-# units: 4 of them, 160 (a second round of 8), 240; contiguous cut: 189 units
+# units: 4 of them, 160 (a second round of 8), 240; contiguous cut: 189 units;
+# clusters of 3, of 6 at hd 128; 4 units split 15 ways
 @pytest.mark.parametrize("Lq,Lk,H,hd", [(840, 2520, 4, 64), (130, 5000, 1, 128), (2196, 3000, 10, 64),
                                         (300, 300, 1, 128), (100, 77, 4, 64), (2500, 500, 16, 128),
-                                        (5000, 129, 12, 64), (2100, 2600, 21, 64)])
+                                        (5000, 129, 12, 64), (2100, 2600, 21, 64),
+                                        (1400, 1000, 7, 64), (840, 2520, 6, 128), (300, 9000, 2, 128)])
 @pytest.mark.parametrize("workspace", ["auto", None])
 def test_attention_orders(Lq, Lk, H, hd, workspace):
     d = H * hd
