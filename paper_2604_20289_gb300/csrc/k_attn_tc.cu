@@ -196,8 +196,8 @@ template <int HD, int ORDER>
 __global__ void __launch_bounds__(352, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO, const int Lq,
-                   const int n_keys, const AttnSplit sp, bf16 *__restrict__ o, const int d, float *__restrict__ ws_o,
-                   float2 *__restrict__ ws_ml, const uint8_t *__restrict__ skip_flag, int *err) {
+                   const int n_keys, const AttnSplit sp, float *__restrict__ ws_o, float2 *__restrict__ ws_ml,
+                   const uint8_t *__restrict__ skip_flag, int *err, bf16 *__restrict__ o, const int d) {
     constexpr bool WAVE = ORDER != ORDER_CONTIGUOUS, CLUSTER = ORDER == ORDER_CLUSTER;
     pdl_wait();
     using A = AttnTile<HD>;
@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(352, 1)
     uint64_t *pv_done = p_full + 2;            // [2] P_i V done (hd 64: every tile; hd 128: last of a piece)
     uint64_t *o_free = pv_done + 2;            // [2] O_i of piece p read out (phase p)
     uint64_t *turn = o_free + 2;               // [2][4] exponential-phase hand-off per (WG, quadrant)
-    uint64_t *all_pv = turn + 8;               // clusters: every P V of the CTA done (its K / V ring is free)
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(all_pv + 1);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(turn + 8);
+    uint64_t *all_pv = turn + 9;               // clusters: every P V of the CTA done (its K / V ring is free)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkt = sp.n_kt;
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(352, 1)
     if (threadIdx.x == 0) {
         mbar_init(q_full, 1);
         mbar_init(q_empty, A::ISSUERS);
-        mbar_init(all_pv, 256);
+        if constexpr (CLUSTER) mbar_init(all_pv, 256);
         for (int s = 0; s < A::STAGES; ++s) {
             mbar_init(&k_full[s], 1);
             mbar_init(&k_empty[s], A::ISSUERS);   // freed by every MMA warp
@@ -937,7 +937,7 @@ static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, co
     float *ws_o = n_combine > 0 ? reinterpret_cast<float *>(ws) : nullptr;
     float2 *ws_ml = n_combine > 0 ? reinterpret_cast<float2 *>(ws_o + 2 * ((size_t)n_sm + 1) * 256 * HD) : nullptr;
     e = launch_pdl_cluster(attn_tc_kernel<HD, ORDER>, (unsigned)cluster, dim3(sp.G), dim3(A::THREADS), A::SMEM_BYTES, st,
-                           tq, tk, tv, to, Lq, n_keys, sp, o, d, ws_o, ws_ml, skip, err);
+                           tq, tk, tv, to, Lq, n_keys, sp, ws_o, ws_ml, skip, err, o, d);
     if (e != cudaSuccess) return e;
     if (n_launched) *n_launched = 1;
     if (n_combine > 0) {
