@@ -666,23 +666,30 @@ cudaError_t rope_table(const RopeArgs &r, cudaStream_t st) {
 // ------------------------------------------------------------------- head
 // Output head (a10): v = round(LN(x) * (1 + scale) + shift) W_out + b,
 // W_out [d][16].  CTA = 32 rows, 256 threads.  Pass 1: warp w reduces the
-// moments of rows 4w..4w+3 (two loads in flight per lane).  Pass 2 walks the
-// columns in chunks of 128 (the next chunk's loads in flight meanwhile): the
+// moments of rows 4w..4w+3.  Pass 2 walks the columns in chunks of 128: the
 // CTA writes the modulated chunk h (rounded to the storage type) to shared
 // memory transposed, hT[k][row] (lane = row when staging, so the stores are
 // conflict-free), and the chunk's 128 x 16 block of W_out beside it; warp w
 // then takes keys 16w..16w+15 of the chunk, lane (r4, c4) accumulating rows
 // 4 r4..4 r4+3 x outputs 4 c4..4 c4+3 from one float4 of hT and one of W_out
-// per key (16 FMA, as 8 packed fp32-pair FMAs, per two shared loads).  The 8 warps' partial sums are
-// added in shared memory at the end, in warp order.
+// per key (16 FMA, as 8 packed fp32-pair FMAs, per two shared loads).  The 8
+// warps' partial sums are added in shared memory at the end, in warp order.
+// Bound by the latency of its loads on few CTAs and by issue on many: x, W_out
+// and the modulation of a chunk are loaded while the one before is computed
+// (W_out and the modulation loaded in place before: 12960 x 5120 163 -> 149
+// us, 12960 x 1536 49.5 -> 47.6).  DEEP: the moments take a run of all four
+// rows at a time, the first chunk already in flight, instead of two runs of
+// one row (630 x 512 17.8 -> 11.4 us, 8064 x 512 18.1 -> 15.2; cold caches);
+// its 118 to 128 registers leave two CTAs on an SM instead of three, so it
+// serves grids that need no third (12960 x 5120 DEEP: some 199 us).
 __device__ __forceinline__ void fma4(float2 (&a)[2], float h, const float4 &w) {
     const float2 hh = make_float2(h, h);
     a[0] = __ffma2_rn(hh, make_float2(w.x, w.y), a[0]);
     a[1] = __ffma2_rn(hh, make_float2(w.z, w.w), a[1]);
 }
 constexpr int HEAD_ROWS = 32, HEAD_CH = 128, HEAD_LD = HEAD_ROWS + 4;
-template <typename T>
-__global__ void __launch_bounds__(256)
+template <typename T, bool DEEP>
+__global__ void __launch_bounds__(256, DEEP ? 2 : 3)
     head_kernel(const T *__restrict__ x, const float *__restrict__ hm, const float *__restrict__ w,
                 const float *__restrict__ b, float *__restrict__ v, int L, int d, float eps) {
     pdl_wait();
@@ -690,9 +697,34 @@ __global__ void __launch_bounds__(256)
     __shared__ __align__(16) float hT[HEAD_CH * HEAD_LD];
     __shared__ __align__(16) float ws[HEAD_CH * 16];
     __shared__ float2 stats[HEAD_ROWS];
+    __shared__ __align__(16) float mod[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int row0 = blockIdx.x * HEAD_ROWS;
     const int runs = d / 16;
+    const float *shift = hm, *scale = hm + d;
+    // warp w stages keys [16 w, 16 w + 16) of each chunk for its lane's row;
+    // a chunk's values, its rows of W_out and its modulation (lanes 0-15 the
+    // scales, 16-31 the shifts of the warp's keys) are loaded while the one
+    // before is computed, the first chunk's during the moments
+    const int my_row = row0 + lane, k16 = warp * 16;
+    float xn[16], mn;
+    float4 wn[2];
+    auto fetch = [&](int c0) {
+        if (my_row < L && c0 + k16 < d) {
+            load16<T>(x + (size_t)my_row * d + c0 + k16, xn);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) xn[i] = 0.0f;
+        }
+        mn = c0 + k16 < d ? (lane < 16 ? scale : shift)[c0 + k16 + (lane & 15)] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int q = threadIdx.x + 256 * i;              // float4 of the chunk's 128 x 16 block
+            wn[i] = c0 * 4 + q < d * 4 ? reinterpret_cast<const float4 *>(w)[c0 * 4 + q]
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    if constexpr (DEEP) fetch(0);
     // moments of one 16-element run, merged into mo
     auto add_run = [](Moments &mo, const float (&t)[16]) {
         float sum = 0.0f;
@@ -703,57 +735,66 @@ __global__ void __launch_bounds__(256)
         for (int i = 0; i < 16; ++i) m1.m2 += (t[i] - m1.mean) * (t[i] - m1.mean);
         mo = merge(mo, m1);
     };
-    for (int rr = 0; rr < 4; ++rr) {
-        const int r = warp * 4 + rr, row = row0 + r;
-        Moments mo{0.0f, 0.0f, 0.0f};
-        if (row < L) {
-            const T *xr = x + (size_t)row * d;
-            int run = lane;
-            for (; run + 32 < runs; run += 64) {         // two runs in flight
-                float t0[16], t1[16];
-                load16<T>(xr + 16 * run, t0);
-                load16<T>(xr + 16 * (run + 32), t1);
-                add_run(mo, t0);
-                add_run(mo, t1);
+    if constexpr (DEEP) {
+        Moments mo[4];
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) mo[rr] = Moments{0.0f, 0.0f, 0.0f};
+        for (int run = lane; run < runs; run += 32) {             // the four rows' loads in flight
+            float t[4][16];
+#pragma unroll
+            for (int rr = 0; rr < 4; ++rr) {
+                const int row = min(row0 + warp * 4 + rr, L - 1);
+                load16<T>(x + (size_t)row * d + 16 * run, t[rr]);
             }
-            if (run < runs) {
-                float t0[16];
-                load16<T>(xr + 16 * run, t0);
-                add_run(mo, t0);
-            }
+#pragma unroll
+            for (int rr = 0; rr < 4; ++rr) add_run(mo[rr], t[rr]);
         }
-        mo = warp_moments(mo);
-        if (lane == 0) stats[r] = make_float2(mo.mean, rsqrtf(mo.m2 / (float)d + eps));
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) {
+            mo[rr] = warp_moments(mo[rr]);
+            if (lane == 0) stats[warp * 4 + rr] = make_float2(mo[rr].mean, rsqrtf(mo[rr].m2 / (float)d + eps));
+        }
+    } else {
+        for (int rr = 0; rr < 4; ++rr) {
+            const int r = warp * 4 + rr, row = row0 + r;
+            Moments mo{0.0f, 0.0f, 0.0f};
+            if (row < L) {
+                const T *xr = x + (size_t)row * d;
+                int run = lane;
+                for (; run + 32 < runs; run += 64) {          // two runs in flight
+                    float t0[16], t1[16];
+                    load16<T>(xr + 16 * run, t0);
+                    load16<T>(xr + 16 * (run + 32), t1);
+                    add_run(mo, t0);
+                    add_run(mo, t1);
+                }
+                if (run < runs) {
+                    float t0[16];
+                    load16<T>(xr + 16 * run, t0);
+                    add_run(mo, t0);
+                }
+            }
+            mo = warp_moments(mo);
+            if (lane == 0) stats[r] = make_float2(mo.mean, rsqrtf(mo.m2 / (float)d + eps));
+        }
+        fetch(0);
     }
     __syncthreads();
-    const float *shift = hm, *scale = hm + d;
     const int r4 = lane >> 2, c4 = lane & 3;
     float2 acc[4][2];                                     // [row][column pair]
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
-    const int my_row = row0 + lane;
     const float2 my_st = stats[lane];
-    // warp w stages keys [16 w, 16 w + 16) of each chunk for its lane's row;
-    // the next chunk's values are loaded while the current one is computed
-    float xn[16];
-    auto fetch = [&](int c0) {
-        if (my_row < L && c0 + warp * 16 < d) {
-            load16<T>(x + (size_t)my_row * d + c0 + warp * 16, xn);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) xn[i] = 0.0f;
-        }
-    };
-    fetch(0);
     for (int c0 = 0; c0 < d; c0 += HEAD_CH) {
         const int n = d - c0 < HEAD_CH ? d - c0 : HEAD_CH;      // multiple of 16
-        const int k16 = warp * 16;
+        mod[warp][lane] = mn;
+        __syncwarp();
         if (k16 < n) {
             float t[16];
             if (my_row < L) {
                 float sc[16], sh[16];
-                load16<float>(scale + c0 + k16, sc);
-                load16<float>(shift + c0 + k16, sh);
+                load16<float>(mod[warp], sc);
+                load16<float>(mod[warp] + 16, sh);
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
                     t[i] = round_to<T>((xn[i] - my_st.x) * my_st.y * (1.0f + sc[i]) + sh[i]);
@@ -764,8 +805,8 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
             for (int i = 0; i < 16; ++i) hT[(k16 + i) * HEAD_LD + lane] = t[i];
         }
-        for (int i = threadIdx.x; i < n * 4; i += blockDim.x)
-            reinterpret_cast<float4 *>(ws)[i] = reinterpret_cast<const float4 *>(w + (size_t)c0 * 16)[i];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) reinterpret_cast<float4 *>(ws)[threadIdx.x + 256 * i] = wn[i];
         __syncthreads();
         if (c0 + HEAD_CH < d) fetch(c0 + HEAD_CH);
         const int k_end = 16 * warp + 16 < n ? 16 * warp + 16 : n;
@@ -802,14 +843,16 @@ __global__ void __launch_bounds__(256)
 
 template <typename T>
 cudaError_t head(const T *x, const float *hm, const float *w, const float *b, float *v, int L, int d, float eps,
-                 cudaStream_t st) {
+                 int n_sm, cudaStream_t st) {
     if (d % 16 != 0) return cudaErrorInvalidValue;
-    return launch_pdl(head_kernel<T>, dim3((L + HEAD_ROWS - 1) / HEAD_ROWS), dim3(256), 0, st, x, hm, w, b, v, L, d, eps);
+    const int grid = (L + HEAD_ROWS - 1) / HEAD_ROWS;
+    return launch_pdl(grid <= 2 * n_sm ? head_kernel<T, true> : head_kernel<T, false>, dim3(grid), dim3(256), 0, st, x,
+                      hm, w, b, v, L, d, eps);
 }
 template cudaError_t head<float>(const float *, const float *, const float *, const float *, float *, int, int, float,
-                                 cudaStream_t);
+                                 int, cudaStream_t);
 template cudaError_t head<bf16>(const bf16 *, const float *, const float *, const float *, float *, int, int, float,
-                                cudaStream_t);
+                                int, cudaStream_t);
 
 // --------------------------------------------------------- weight layout
 // Wt[n][k] = convert(W[k][n]) for one [K][N] float32 matrix (32x32 tiles).

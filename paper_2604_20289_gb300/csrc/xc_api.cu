@@ -826,7 +826,7 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
                chain_apply<T>(X[0], X[1], reinterpret_cast<const T *>(ctx->rhat) + (size_t)t * B * Ld, ctx->flags, B,
                               B, (long)Ld, ctx->n_sm, st));
     if (!kv_tail_off)
-        LAUNCH(XC_K_HEAD, -1, 1, head<T>(X[B & 1], ctx->hmod, ctx->out_w, ctx->out_b, v_dev, L, d, ctx->cfg.ln_eps, st));
+        LAUNCH(XC_K_HEAD, -1, 1, head<T>(X[B & 1], ctx->hmod, ctx->out_w, ctx->out_b, v_dev, L, d, ctx->cfg.ln_eps, ctx->n_sm, st));
     };   // body
 
     if (ctx->prof_on || !ctx->graphs_on) {

@@ -143,7 +143,7 @@ struct CondArgs {
 cudaError_t conditioning(const CondArgs &c, cudaStream_t st);
 template <typename T>
 cudaError_t head(const T *x, const float *hm, const float *w, const float *b, float *v, int L, int d, float eps,
-                 cudaStream_t st);
+                 int n_sm, cudaStream_t st);
 template <typename T> cudaError_t transpose_convert(const float *W, T *Wt, int K, int N, cudaStream_t st);
 cudaError_t rope_table(const RopeArgs &r, cudaStream_t st);
 // Test of the bounded waits: a one-thread kernel whose wait runs out (after
