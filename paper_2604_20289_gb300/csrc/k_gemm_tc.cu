@@ -9,6 +9,8 @@
 //          own with a 128 x 256 tile loads 48 KB -- the operand feed from L2
 //          bounds the main loop, so a third fewer bytes per MMA is what the
 //          pair is for (and six ring stages fit instead of four);
+//   wide   (BN = 256, WIDE) one CTA per 128 x 256 tile, four ring stages, where
+//          the row count leaves the pairs a ragged last round;
 //   single (BN = 128, 64) one CTA per 128 x BN tile, for GEMMs with too few
 //          256 x 256 tiles to fill the pairs.  With few tiles a k step waits
 //          for the latency of its loads (some 2200 cycles over the ring's
@@ -55,7 +57,7 @@ constexpr int EPI_BLOCK_BYTES = 32 * 32 * 2;   // one 32 x 32 bf16 block
 // residual operands of a block land in its slot AHEAD blocks before they are
 // needed, the output replaces them in place (a lane touches its own row
 // only), and a slot is loaded or written again once its store has been read.
-template <int BN, int EPI, bool DEEP>
+template <int EPI, bool DEEP, bool WIDE>
 struct EpiRing {
     static constexpr bool RES = EPI == EPI_RESID_GATE || EPI == EPI_RESID_CACHE;
     static constexpr bool CACHE = EPI == EPI_RESID_CACHE;
@@ -63,20 +65,22 @@ struct EpiRing {
     // residual with a short K gains more from loading two blocks ahead.  Two /
     // four slots measured: 8064 x 1536 x 512 13.3 / 14.4 us, 12960 x 8960 x
     // 1536 + GELU 187 / 190; gated 6000 x 4096 x 512 28.0 / 25.9, gated 4000
-    // x 256 x 6976 23.9 / 26.6
-    static constexpr int SLOTS = DEEP ? 4 : 2;
+    // x 256 x 6976 23.9 / 26.6.  A wide tile's residual cache has room for one
+    // (loaded when its block begins) beside four main-loop stages: one slot and
+    // four stages / two and three at 2356 x 2048 x 3392 24.0 / 28.6
+    static constexpr int SLOTS = DEEP ? 4 : WIDE && CACHE ? 1 : 2;
     static constexpr int AHEAD = SLOTS / 2;
     static constexpr int SLOT_BYTES = (CACHE ? 2 : 1) * EPI_BLOCK_BYTES;
 };
 
-template <int BN, int EPI, bool DEEP>
+template <int BN, int EPI, bool DEEP, bool WIDE>
 struct GemmTile {
-    static constexpr bool PAIR = BN == 256;            // two CTAs per tile
+    static constexpr bool PAIR = BN == 256 && !WIDE;   // two CTAs per tile
     static constexpr int BM = PAIR ? 2 * GEMM_BM : GEMM_BM;
     static constexpr int A_BYTES = GEMM_BM * GEMM_BK * 2;
     static constexpr int B_BYTES = (PAIR ? 128 : BN) * GEMM_BK * 2;   // pair: this CTA's half of B's rows
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int EPI_BYTES = 8 * EpiRing<BN, EPI, DEEP>::SLOTS * EpiRing<BN, EPI, DEEP>::SLOT_BYTES;
+    static constexpr int EPI_BYTES = 8 * EpiRing<EPI, DEEP, WIDE>::SLOTS * EpiRing<EPI, DEEP, WIDE>::SLOT_BYTES;
     static constexpr int VEC_BYTES = 8 * 64 * 4;       // bias and gate of a warp's block
     static constexpr int BAR_BYTES = VEC_BYTES + 512;
     static constexpr int FIT = (GEMM_SMEM_LIMIT - BAR_BYTES - EPI_BYTES) / STAGE_BYTES;
@@ -193,15 +197,15 @@ __device__ __forceinline__ Tile tile_at(const TileWalk &tw, int item) {
     return r;
 }
 
-template <int BN, int EPI, bool DEEP>
+template <int BN, int EPI, bool DEEP, bool WIDE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ WeightMaps tmB,
                    const __grid_constant__ EpiMaps em, const EpiParams ep, const int K, const TileWalk tw,
                    const uint8_t *__restrict__ skip_flag, int *err) {
-    using G = GemmTile<BN, EPI, DEEP>;
+    using G = GemmTile<BN, EPI, DEEP, WIDE>;
     if (threadIdx.x == 0) {                           // kernel parameters: nothing a predecessor writes
         prefetch_tmap(&tmA);
-        prefetch_tmap(BN == 64 ? &tmB.box64 : &tmB.box128);
+        prefetch_tmap(WIDE ? &tmB.box256 : BN == 64 ? &tmB.box64 : &tmB.box128);
     }
     pdl_wait();
     if (skip_flag != nullptr && *skip_flag == XC_DEC_SKIP) return;
@@ -217,7 +221,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     uint64_t *acc_full = empty + G::STAGES;    // [2]
     uint64_t *acc_empty = acc_full + 2;        // [2]
     uint64_t *ld_bar = acc_empty + 2;          // [8][SLOTS] residual operands of an epilogue warp's slot landed
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ld_bar + 8 * EpiRing<BN, EPI, DEEP>::SLOTS);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ld_bar + 8 * EpiRing<EPI, DEEP, WIDE>::SLOTS);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KT = K / GEMM_BK;
@@ -236,7 +240,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], G::EPI_WARPS);
         }
-        for (int w = 0; w < 8 * EpiRing<BN, EPI, DEEP>::SLOTS; ++w) mbar_init(&ld_bar[w], 1);
+        for (int w = 0; w < 8 * EpiRing<EPI, DEEP, WIDE>::SLOTS; ++w) mbar_init(&ld_bar[w], 1);
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -257,7 +261,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             const Tile t = tile_at<G::BM, BN>(tw, item);
             const int m0 = t.m0 + row_off, n0 = PAIR ? t.n0 + (int)rank * (t.w / 2) : t.n0;
             const int b_rows = PAIR ? t.w / 2 : BN;           // of B
-            const CUtensorMap *tb = b_rows == 128 ? &tmB.box128 : &tmB.box64;
+            const CUtensorMap *tb = WIDE ? &tmB.box256 : b_rows == 128 ? &tmB.box128 : &tmB.box64;
             const uint32_t bytes = (uint32_t)G::A_BYTES + (uint32_t)b_rows * (GEMM_BK * 2);
             for (int kt = 0; kt < KT; ++kt, ++it) {
                 const int s = it % G::STAGES;
@@ -333,7 +337,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         // ---------------------------------------------------------- epilogue (warps 2..9)
         // Warp ew = warp - 2 owns TMEM lane quadrant q (rows q*32 .. q*32+31 of
         // the tile; thread = row) and column half `half`, in 32-column blocks.
-        using E = EpiRing<BN, EPI, DEEP>;
+        using E = EpiRing<EPI, DEEP, WIDE>;
         const int ew = warp - 2;
         const int q = warp & 3;
         const int half = ew >> 2;
@@ -620,7 +624,7 @@ template <int EPI, bool DEEP>
 static int pair_count() {
     static int n = 0;
     if (n == 0) {
-        using G = GemmTile<256, EPI, DEEP>;
+        using G = GemmTile<256, EPI, DEEP, false>;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2 * (gemm_sm_count() / 2));
         cfg.blockDim = dim3(GEMM_THREADS);
@@ -633,7 +637,7 @@ static int pair_count() {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int k = 0;
-        if (cudaOccupancyMaxActiveClusters(&k, gemm_tc_kernel<256, EPI, DEEP>, &cfg) != cudaSuccess || k < 1) {
+        if (cudaOccupancyMaxActiveClusters(&k, gemm_tc_kernel<256, EPI, DEEP, false>, &cfg) != cudaSuccess || k < 1) {
             cudaGetLastError();
             k = gemm_sm_count() / 2;
         }
@@ -654,37 +658,46 @@ static TileWalk pair_walk(int M, int N, int workers) {
     return tw;
 }
 
-// Output tiling for an M x N x K GEMM: 256 (CTA pairs), 128 or 64 (single
-// CTAs).  Half the pairs' worth of 256 x 256 tiles and fewer are one round of
-// single tiles, 64 wide while those find an SM each.  Beyond, the cost in SM
-// cycles of the persistent rounds: a 64-deep k step takes about 555 cycles
-// on a full pair tile, 340 on a half one, 450 on a single tile with every SM
-// busy (bound by its operand feed); no round is shorter than its epilogue,
-// the last one's is added, and setting up a pair takes some 1500 more.
-// Measured, pair / 128-wide single: 8064 x 512 x 512 8.5 / 7.6 us, 840 x 1024
-// x 256 7.3 / 4.6, 8064 x 2048 x 512 + GELU 16.6 / 18.1, 700 x 5120 x 1024 +
-// residual cache 17.6 / 14.3, 239 x 12032 x 3712 22.0 / 27.7, 1554 x 6144 x
-// 11072 142 / 176, 12960 x 5120 x 5120 366 / 498.
+// Output tiling for an M x N x K GEMM: 256 (CTA pairs), GEMM_WIDE, 128 or 64
+// (single CTAs).  Half the pairs' worth of 256 x 256 tiles and fewer are one
+// round of single tiles, 64 wide while those find an SM each.  Beyond, the cost
+// in SM cycles of the persistent rounds: a 64-deep k step takes about 555
+// cycles on a full pair tile, 340 on a half one, 640 on a wide single tile, 450
+// on a 128-wide one with every SM busy (bound by the operand feed); no round is
+// shorter than its epilogue, the last one's is added, and setting up a pair
+// takes some 1500 more, 3500 where a few row blocks make most of B a tile's
+// own.  Wide tiles are for row counts that leave the pairs a ragged round.
+// Measured, pair / wide / 128-wide: gated residual 2356 x 2048 x 3392 30.7 /
+// 20.5 / 24.4 us, 1900 x 2560 x 6144 52.3 / 37.3 / 40.5, 500 x 9728 x 1536 13.4
+// / 12.3 / 13.7, 4800 x 4096 x 2048 47.6 / 52.8 / 60.1, 12960 x 5120 x 5120 363 /
+// 411 / 453, 9728 x 512 x 512 8.6 / 7.8 / 7.7; residual cache 2356 x 2048 x 3392
+// 33.2 / 24.0 / 27.1, x 1024 16.6 / 13.3 / 12.6, 7200 x 2560 x 1024 40.5 / 43.7 /
+// 48.7; 239 x 12032 x 3712 22.0 / - / 27.7.
 int gemm_tc_bn(int epi, int M, int N, int K) {
     const long n_sm = gemm_sm_count(), pairs = n_sm / 2 < 1 ? 1 : n_sm / 2;
-    const long t128 = (long)((M + 127) / 128) * (N / 128), r128 = (t128 + n_sm - 1) / n_sm;
+    const long tm = (M + 127) / 128, t128 = tm * (N / 128), r128 = (t128 + n_sm - 1) / n_sm;
     if (2 * t128 <= n_sm) return 64;
     if (N % 256 != 0) return 128;
     const TileWalk tw = pair_walk(M, N, (int)pairs);
     if (tw.n_full == 0) return 128;
     const long r_full = (tw.n_full + pairs - 1) / pairs, r_half = tw.n_items > tw.n_full ? 1 : 0;
+    const long r_wide = (tm * (N / 256) + n_sm - 1) / n_sm;
     const long kt = K / GEMM_BK;
     const long e_full = epi == EPI_RESID_CACHE ? 12000 : 4500, e_half = epi == EPI_RESID_CACHE ? 6000 : 2500;
     const long pair = r_full * std::max(kt * 555, e_full) + r_half * std::max(kt * 340, e_half) +
-                      (r_half ? e_half : e_full) + 1500;
-    return pair <= r128 * std::max(kt * 450, e_half) + e_half ? 256 : 128;
+                      (r_half ? e_half : e_full) + (tw.tiles_m <= 4 ? 3500 : 1500);
+    const long e_wide = epi == EPI_RESID_CACHE ? 14000 : 4500;
+    const long wide = r_wide * std::max(kt * 640, e_wide) + e_wide;
+    const long narrow = r128 * std::max(kt * 450, e_half) + e_half;
+    if (wide < pair && 20 * wide < 19 * narrow) return GEMM_WIDE;
+    return pair <= narrow ? 256 : 128;
 }
 
-template <int EPI, int BN, bool DEEP = false>
+template <int EPI, int BN, bool DEEP = false, bool WIDE = false>
 static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                              const uint8_t *skip, int *err, cudaStream_t st) {
-    using G = GemmTile<BN, EPI, DEEP>;
-    auto kern = gemm_tc_kernel<BN, EPI, DEEP>;
+    using G = GemmTile<BN, EPI, DEEP, WIDE>;
+    auto kern = gemm_tc_kernel<BN, EPI, DEEP, WIDE>;
     EpiMaps em;
     if (!build_epi_maps<EPI>(em, ep)) return cudaErrorInvalidValue;
     static bool attr_set = false;
@@ -708,27 +721,28 @@ static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const 
                               ta, tb, em, ep, K, tw, skip, err);
 }
 
-template <int BN>
+template <int BN, bool WIDE = false>
 static cudaError_t gemm_tc_bn_(int epi, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                                const uint8_t *skip, int *err, cudaStream_t st) {
     switch (epi) {
-        case EPI_BIAS: return launch_tc<EPI_BIAS, BN>(ta, tb, ep, K, skip, err, st);
-        case EPI_GELU: return launch_tc<EPI_GELU, BN>(ta, tb, ep, K, skip, err, st);
+        case EPI_BIAS: return launch_tc<EPI_BIAS, BN, false, WIDE>(ta, tb, ep, K, skip, err, st);
+        case EPI_GELU: return launch_tc<EPI_GELU, BN, false, WIDE>(ta, tb, ep, K, skip, err, st);
         case EPI_RESID_GATE:
-            if constexpr (BN == 64) return launch_tc<EPI_RESID_GATE, BN>(ta, tb, ep, K, skip, err, st);
-            return K < 1536 ? launch_tc<EPI_RESID_GATE, BN, true>(ta, tb, ep, K, skip, err, st)
-                            : launch_tc<EPI_RESID_GATE, BN>(ta, tb, ep, K, skip, err, st);
-        case EPI_RESID_CACHE: return launch_tc<EPI_RESID_CACHE, BN>(ta, tb, ep, K, skip, err, st);
-        case EPI_QKV_ROPE: return launch_tc<EPI_QKV_ROPE, BN>(ta, tb, ep, K, skip, err, st);
+            if constexpr (BN == 64 || WIDE) return launch_tc<EPI_RESID_GATE, BN, false, WIDE>(ta, tb, ep, K, skip, err, st);
+            else return K < 1536 ? launch_tc<EPI_RESID_GATE, BN, true>(ta, tb, ep, K, skip, err, st)
+                                 : launch_tc<EPI_RESID_GATE, BN>(ta, tb, ep, K, skip, err, st);
+        case EPI_RESID_CACHE: return launch_tc<EPI_RESID_CACHE, BN, false, WIDE>(ta, tb, ep, K, skip, err, st);
+        case EPI_QKV_ROPE: return launch_tc<EPI_QKV_ROPE, BN, false, WIDE>(ta, tb, ep, K, skip, err, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
 // Entry used by the chunk step and xc_op_linear / xc_op_qkv_rope (bf16 only).
 // `ta` covers A [M][K] (boxes of 128 rows), `tb` Wt [N][K]; bn =
-// gemm_tc_bn(epi, M, N, K); N % bn == 0, K % 64 == 0.
+// gemm_tc_bn(epi, M, N, K); N a multiple of the tile's width, K % 64 == 0.
 cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                     const uint8_t *skip, int *err, cudaStream_t st) {
+    if (bn == GEMM_WIDE) return gemm_tc_bn_<256, true>(epi, ta, tb, ep, K, skip, err, st);
     if (bn == 256) return gemm_tc_bn_<256>(epi, ta, tb, ep, K, skip, err, st);
     if (bn == 128) return gemm_tc_bn_<128>(epi, ta, tb, ep, K, skip, err, st);
     if (bn == 64) return gemm_tc_bn_<64>(epi, ta, tb, ep, K, skip, err, st);

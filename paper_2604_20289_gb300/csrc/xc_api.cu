@@ -34,7 +34,7 @@ struct Fail {
 
 // RoPE pair table: head_dim split hd/8 (camera) : 3hd/8 (absolute frame) :
 // hd/4 (h) : hd/4 (w); pair j of an axis with D dims rotates at theta^(-2j/D).
-// For the per-chunk (cos, sin) table (rope_table_kernel): the axis of every
+// For the per-chunk (cos, sin) table (rope_entry): the axis of every
 // pair and the table entry of its position 0; npos = positions per axis
 // (cameras, frames per chunk, h, w).  Returns the number of table entries.
 int rope_layout(int hd, const int npos[4], std::vector<int> &axis, std::vector<int> &off) {
@@ -455,6 +455,7 @@ void tmap(xc_ctx *ctx, CUtensorMap *m, const void *base, uint64_t rows, uint64_t
 void wmap(xc_ctx *ctx, WeightMaps *m, const void *base, uint64_t rows, uint64_t cols) {
     tmap(ctx, &m->box128, base, rows, cols, 128);
     tmap(ctx, &m->box64, base, rows, cols, 64);
+    tmap(ctx, &m->box256, base, rows, cols, 256);
 }
 
 // Profiling hooks: an event pair around one launch when its kind is selected.

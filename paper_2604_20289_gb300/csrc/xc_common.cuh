@@ -154,7 +154,7 @@ struct EpiParams {
         g_gw[XC_MAX_GROUPS];
     const int *rope_axis;      // [head_dim/2] 0 camera, 1 frame, 2 h, 3 w
     const int *rope_off;       // [head_dim/2] table entry of position 0 of each pair
-    const float2 *rope_cs;     // (cos, sin) table of this chunk (rope_table_kernel)
+    const float2 *rope_cs;     // (cos, sin) table of this chunk (rope_entry)
 };
 
 // One view group covering every camera (grid gh x gw).

@@ -87,15 +87,20 @@ template <typename T>
 cudaError_t chain_apply(T *x0, T *x1, const T *rhat_t, const uint8_t *flags, int b, int n_blocks, long ld,
                         int n_sm, cudaStream_t st);
 bool make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows);
-// A weight matrix Wt [N][K] of the bf16 GEMM, in boxes of 128 rows and, for
-// the half tiles of a last round, of 64.
+// A weight matrix Wt [N][K] of the bf16 GEMM, in boxes of 128 rows, of 64 for
+// the half tiles of a last round and narrow tiles, of 256 for wide single ones.
 struct WeightMaps {
-    CUtensorMap box128, box64;
+    CUtensorMap box128, box64, box256;
 };
+// Tiling of gemm_tc_bn: 64, 128 (single CTAs), 256 (CTA pairs), GEMM_WIDE
+// (single CTAs, 256 columns).
+constexpr int GEMM_WIDE = 257;
 // The maps that tiling bn uses (0: all).
 inline bool make_weight_maps(WeightMaps *m, int bn, const void *base, uint64_t N, uint64_t K) {
-    if (bn != 64 && !make_tmap_bf16(&m->box128, base, N, K, 128)) return false;
-    return bn == 128 || make_tmap_bf16(&m->box64, base, N, K, 64);
+    const bool all = bn == 0;
+    return (!(all || bn == 128 || bn == 256) || make_tmap_bf16(&m->box128, base, N, K, 128)) &&
+           (!(all || bn == 64 || bn == 256) || make_tmap_bf16(&m->box64, base, N, K, 64)) &&
+           (!(all || bn == GEMM_WIDE) || make_tmap_bf16(&m->box256, base, N, K, 256));
 }
 int gemm_tc_bn(int epi, int M, int N, int K);
 cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,

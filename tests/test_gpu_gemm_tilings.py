@@ -1,5 +1,5 @@
 """The bf16 GEMM's tilings -- CTA pairs (256 x 256 tiles, halves in a short
-last round), single CTAs with 128- and 64-wide tiles -- at the sizes where
+last round), single CTAs with 256-, 128- and 64-wide tiles -- at the sizes where
 they can go wrong: a second CTA without a row of its own, a last row tile of
 few rows, one round without halves, halves beside full tiles, several rounds,
 both staging depths of the gated residual, K below the ring's depth, and the
@@ -45,12 +45,14 @@ def close(t, want):
     assert xb.op_device_error() == 0
 
 
-# M = 2370: 66 rows in the last row tile (none for the second CTA); 2500: 196;
-# 2432: 128 exactly.  N = 1280: one round of full tiles; 2048: 76 + halves;
-# 4096: two rounds + halves.  K = 1024 / 1600: both staging depths.  Then
-# 128-wide single tiles (88 of them) and 64-wide ones
+# M = 2370: 66 rows in the last row tile (none for a pair's second CTA); 2500:
+# 196; 2432: 128 exactly.  N = 1280: one round of full pair tiles; M 2500 N 2048:
+# 76 + halves; N 4096: two rounds + halves.  K = 1024 / 1600: both staging
+# depths.  Wide single tiles: 2432 x 2048 (one round, 152), 2370 x 4096 (two),
+# 2356 x 2048 x 3392 (with the residual cache too).  Then 128-wide single tiles
+# (88 of them) and 64-wide ones
 @pytest.mark.parametrize("M,N,K", [(2370, 1280, 1024), (2500, 2048, 1024), (2432, 2048, 1600), (2370, 4096, 1600),
-                                   (1300, 1024, 64), (1300, 1024, 1600), (130, 512, 128), (1, 256, 1600)])
+                                   (2500, 4096, 1600), (2356, 2048, 3392), (1300, 1024, 64), (1300, 1024, 1600), (130, 512, 128), (1, 256, 1600)])
 @pytest.mark.parametrize("epi", [xb.XC_EPI_BIAS, xb.XC_EPI_GELU, xb.XC_EPI_RESID_GATE, xb.XC_EPI_RESID_CACHE])
 def test_linear_tilings(M, N, K, epi):
     A, Wt = rt(f"A{M}{K}", (M, K)), rt(f"W{N}{K}", (N, K), 1 / math.sqrt(K))
@@ -72,9 +74,11 @@ def test_linear_tilings(M, N, K, epi):
         assert torch.equal(rh[:M], (out[:M].float() - dev(xin).float()).to(torch.bfloat16))
 
 
+# 2550 rows, N = 2304: pairs; 1980 rows: wide single tiles
+@pytest.mark.parametrize("gh,gw", [(17, 25), (15, 22)])
 @pytest.mark.parametrize("hd", [64, 128])
-def test_qkv_rope_pairs(hd):
-    cams, frames, gh, gw, d, chunk = 3, 2, 17, 25, 768, 5        # 2550 rows, N = 2304
+def test_qkv_rope_pairs(hd, gh, gw):
+    cams, frames, d, chunk = 3, 2, 768, 5
     M, H = cams * frames * gh * gw, d // hd
     A, Wt, b = rt(f"qa{hd}", (M, d)), rt(f"qw{hd}", (3 * d, d), 1 / math.sqrt(d)), rt(f"qb{hd}", (3 * d,), 0.1, False)
     q, k, v = (torch.empty(M, d, device=DEV, dtype=torch.bfloat16) for _ in range(3))
