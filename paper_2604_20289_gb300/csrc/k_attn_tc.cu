@@ -26,9 +26,10 @@
 // tile) take turns on the MUFU-bound exponential phase.
 // Online softmax in the exp2 domain with lazy rescaling: a row's O and sum
 // are rescaled only when its running max grows by more than 8 (hd 64), or
-// when a tile's row sum passes 2^40 under the max in use (hd 128).  Score scaling and row sums use packed fp32 pairs
-// (FFMA2 / FADD2).  Keys beyond n_keys (ragged last tile) are masked to -inf;
-// their K/V rows are finite (zero-initialised ring, TMA zero fill).
+// when a tile's row sum passes 2^40 under the max in use (hd 128).  Score
+// scaling and row sums use packed fp32 pairs (FFMA2 / FADD2).  Keys beyond
+// n_keys (ragged last tile) are masked to -inf; their K/V rows are finite
+// (zero-initialised ring, TMA zero fill).
 #include <algorithm>
 
 #include "xc_ptx.cuh"
@@ -118,9 +119,9 @@ __device__ __forceinline__ void exp_quarter(const float (&s)[128], int qt, float
 }
 
 // Work split.  A unit is (head, pair of 128-query tiles), u = head * n_qblk +
-// qblk, with n_kt key tiles, walked by G CTAs (one per SM) in one of two
+// qblk, with n_kt key tiles, walked by G CTAs (one per SM) in one of three
 // orders:
-//  * contiguous (WAVE = false): the (unit, key tile) iteration space, T =
+//  * contiguous (ORDER_CONTIGUOUS): the (unit, key tile) iteration space, T =
 //    n_units * n_kt, is cut into the contiguous shares [c T / G,
 //    (c + 1) T / G).  A unit cut by the boundary between CTAs c - 1 and c is
 //    finished by both as an unnormalised partial O with its running max m
@@ -129,7 +130,7 @@ __device__ __forceinline__ void exp_quarter(const float (&s)[128], int qt, float
 //    unit, so a unit is cut at most once.  The units in flight span every
 //    head, so each unit streams its head's K / V from DRAM once the heads'
 //    K / V exceed L2.
-//  * waves (WAVE = true): CTA c runs the whole units c, c + G, ..., W of
+//  * waves (ORDER_WAVE): CTA c runs the whole units c, c + G, ..., W of
 //    them and one more if c < R -- the CTAs running at one time share a few
 //    heads and each K / V tile comes from DRAM once per wave -- and, where
 //    T2 > 0 (then R = 0), the key tiles of the remaining units, T2 of them,
