@@ -26,7 +26,7 @@
 // tile) take turns on the MUFU-bound exponential phase.
 // Online softmax in the exp2 domain with lazy rescaling: a row's O and sum
 // are rescaled only when its running max grows by more than 8 (hd 64), or
-// when a tile's row sum passes 2^40 under the max in use (hd 128).  Score
+// when a tile's row sum passes 2^15 under the max in use (hd 128).  Score
 // scaling and row sums use packed fp32 pairs (FFMA2 / FADD2).  Keys beyond
 // n_keys (ragged last tile) are masked to -inf; their K/V rows are finite
 // (zero-initialised ring, TMA zero fill).
@@ -57,7 +57,10 @@ struct AttnTile {
     __host__ __device__ static constexpr int O_COL(int i) { return 256 + HD * i; }
     __host__ __device__ static constexpr int P_COL(int i) { return SEP_P ? 256 + 2 * HD + 64 * i : 128 * i; }
     static constexpr float LAZY = 8.0f;                // hd 64: rescale threshold (log2 units)
-    static constexpr float RAISE = 1099511627776.0f;   // hd 128: 2^40, a tile's row sum
+    // hd 128: limit of a tile's row sum, that of 128 keys 2^LAZY above the max in
+    // use, so that O and l have the same range at both head dims: n_kt tiles of
+    // values below 2^112 / n_kt stay finite
+    static constexpr float RAISE = 32768.0f;
 };
 
 __device__ __forceinline__ uint8_t *align1024_a(uint8_t *p) {
@@ -505,7 +508,7 @@ __global__ void __launch_bounds__(352, 1)
                 // hd 128.  m is the row max of the piece's first tile; a later
                 // tile takes it as it is, without a max of its own: bf16 and
                 // fp32 share their exponent range, so scores above m cost no
-                // precision until the sums near overflow.  The tile's row sum
+                // precision while the sums stay small.  The tile's row sum
                 // tells: past RAISE (or not a number) the row's m is raised to
                 // its max, O and l are rescaled, and the tile is done again
                 // from the scores still in registers.  (The commit behind

@@ -1,9 +1,9 @@
 """bf16 attention's work orders at the sizes where they can go wrong: units
 split over several CTAs (evenly, and over all SMs with shares that touch two
 units), whole units in waves with and without a last round, no workspace, a
-second query tile without a row, ragged keys, one key tile; and scores that
+second query tile without a row, ragged keys, one key tile; scores that
 outgrow the running max at head_dim 128, whose later tiles take no max of
-their own.
+their own; and scores of a later tile that are not finite.
 
 Tolerance: the probabilities are rounded to bf16 before P V, 2^-9 relative
 noise averaged over the keys: rel-L2 <= 5e-3 over all rows, 2e-2 for each.
@@ -58,14 +58,43 @@ def test_attention_orders(Lq, Lk, H, hd, workspace):
 
 # Hot keys from the second tile on, each its query's direction times c: the
 # score outgrows the first tile's max by c sqrt(128) / ln 2 in log2 units -- 16 c:
-# 32 (no raise), 80 (raise), 240 (first pass infinite); then growing over tiles
-@pytest.mark.parametrize("c", [2.0, 5.0, 15.0])
+# 14 (no raise), 32 and 80 (raise), 240 (first pass infinite); then growing over
+# tiles.  Values of 2^100 stay finite: a tile's weights sum to at most 2^15, so
+# that the unnormalised output of 12 tiles is below 2^120
+@pytest.mark.parametrize("c,v_scale", [(0.9, 1.0), (2.0, 1.0), (5.0, 1.0), (15.0, 1.0), (0.9, 2.0 ** 100), (2.0, 2.0 ** 100)])
 @pytest.mark.parametrize("workspace", ["auto", None])
-def test_attention_hd128_outgrown_max(c, workspace):
+def test_attention_hd128_outgrown_max(c, v_scale, workspace):
     Lq, Lk, hd = 256, 1500, 128
     q = X.random_tensor(19, "oq", (Lq, hd), bf16=True)
     k = X.random_tensor(19, "ok", (Lk, hd), std=0.05, bf16=True)
-    v = X.random_tensor(19, "ov", (Lk, hd), bf16=True)
+    v = X.random_tensor(19, "ov", (Lk, hd), bf16=True) * np.float32(v_scale)
     for rep, at in ((0.6, 200), (1.0, 700), (0.8, 1200)):    # three hot keys per query, the largest in the middle
         k[at + np.arange(Lq)] = X.bf16_representable((q * c * rep).astype(np.float32))
     check(q, k, v, 1, hd, workspace)
+
+
+# A key with one infinite component in a later tile: its score is -inf for the
+# queries with a negative component there (weight 0) and +inf for the others
+# (not a number, and only in their rows); a key that is not a number takes every row
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("workspace", ["auto", None])
+def test_attention_non_finite_scores_of_a_later_tile(hd, workspace):
+    Lq, Lk, at = 256, 1500, 700
+    q = X.random_tensor(23, "nq", (Lq, hd), bf16=True)
+    k = X.random_tensor(23, "nk", (Lk, hd), bf16=True)
+    v = X.random_tensor(23, "nv", (Lk, hd), bf16=True)
+    assert (q[:, 3] != 0).all()
+    bf = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV).to(torch.bfloat16)   # noqa: E731
+    want = O.to_bf16(O.attention(*(np.delete(a, at if a is not q else [], 0).reshape(-1, 1, hd).astype(np.float64)
+                                   for a in (q, k, v))).reshape(Lq, hd))
+    k[at, 3] = np.inf
+    o = torch.empty(Lq, hd, device=DEV, dtype=torch.bfloat16)
+    xb.op_attention("bf16", 1, hd, bf(q), bf(k), bf(v), o, workspace=workspace)
+    got = o.double().cpu().numpy()
+    hit = q[:, 3] > 0
+    assert np.isnan(got[hit]).all() and np.isfinite(got[~hit]).all()
+    assert np.linalg.norm(got[~hit] - want[~hit]) <= 5e-3 * np.linalg.norm(want[~hit])
+    k[at, 3] = np.nan
+    xb.op_attention("bf16", 1, hd, bf(q), bf(k), bf(v), o, workspace=workspace)
+    assert bool(torch.isnan(o).all())
+    assert xb.op_device_error() == 0
