@@ -52,14 +52,14 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
  * every key: full attention within the chunk and over all resident cached
  * keys).  q, o [Lq][H*hd]; k, v [n_keys][H*hd] (bf16: 16-byte aligned rows).
  *   workspace  device, optional.  With at least
- *              xc_op_attention_workspace_bytes() bytes, the key ranges of
- *              (head, 256-query) units may be split over the SMs: the (unit,
+ *              xc_op_attention_workspace_bytes() bytes, 16-byte aligned, the
+ *              key ranges of (head, 256-query) units may be split over the SMs: the (unit,
  *              key tile) space cut into equal shares; with 8 or more waves of
  *              units and the K / V of all heads larger than L2, whole units in
  *              waves and only the remaining ones cut; with fewer units than
  *              SMs, each over several CTAs.  A second kernel (or the unit's
  *              thread-block cluster) merges the partials.  Short key ranges
- *              run whole all the same.  With NULL (or too small) every
+ *              run whole all the same.  With NULL (too small, not aligned) every
  *              unit runs whole on one SM.  Contents on entry are ignored; it
  *              must not be shared by calls that overlap in time.
  * bf16 needs head_dim 64 or 128; fp32 head_dim 16, 32 or 64. */

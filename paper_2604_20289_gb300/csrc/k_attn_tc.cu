@@ -982,7 +982,9 @@ static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, con
     sp.n_qblk = (Lq + A::QT * A::BQ - 1) / (A::QT * A::BQ);
     const int n_units = sp.n_qblk * n_heads;
     const int n_sm = sm_count();
-    const bool can_cut = ws != nullptr && ws_bytes >= attn_workspace_bytes(HD);
+    // (partials leave by bulk copies: 16-byte aligned)
+    const bool can_cut = ws != nullptr && ws_bytes >= attn_workspace_bytes(HD) &&
+                         (reinterpret_cast<uintptr_t>(ws) & 15) == 0;
     sp.T = (long long)n_units * sp.n_kt;
     sp.T2 = 0;
     sp.G = n_units < n_sm ? n_units : n_sm;
@@ -1042,7 +1044,8 @@ static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, con
 
 // q [Lq][d], k / v maps over [>= n_keys][d] (boxes of 128 rows), o [Lq][d] and
 // its map (boxes of 32 rows); hd in {64, 128}.  ws: attn_workspace_bytes(hd)
-// bytes let units be cut between CTAs (nullptr: whole units only).
+// bytes, 16-byte aligned, let units be cut between CTAs (nullptr, smaller or
+// not aligned: whole units only).
 cudaError_t attn_tc(int head_dim, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
                     const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes,
                     const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {

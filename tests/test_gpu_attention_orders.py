@@ -56,6 +56,18 @@ def test_attention_orders(Lq, Lk, H, hd, workspace):
     check(q, k, v, H, hd, workspace)
 
 
+# A workspace that is not 16-byte aligned is not used (units whole): units that
+# would be split 15 ways, cut contiguously, in a cluster
+@pytest.mark.parametrize("Lq,Lk,H,hd", [(300, 9000, 2, 128), (2100, 2600, 21, 64), (840, 2520, 4, 64)])
+def test_attention_workspace_alignment(Lq, Lk, H, hd):
+    d = H * hd
+    q, k, v = (X.random_tensor(17, n + f"{r}x{d}", (r, d), std=s, bf16=True)
+               for n, r, s in (("q", Lq, 1.5), ("k", Lk, 1.0), ("v", Lk, 1.0)))
+    ws = torch.zeros(xb.op_attention_workspace_bytes("bf16", hd) + 16, dtype=torch.uint8, device=DEV)
+    check(q, k, v, H, hd, ws[8:])
+    assert int(ws.sum()) == 0
+
+
 # Hot keys from the second tile on, each its query's direction times c: the
 # score outgrows the first tile's max by c sqrt(128) / ln 2 in log2 units -- 16 c:
 # 14 (no raise), 32 and 80 (raise), 240 (first pass infinite); then growing over
