@@ -42,7 +42,9 @@ xc_status xc_op_linear(int dtype, int epilogue, int M, int N, int K, const void 
  * (camera, absolute frame, h, w)).  A [M][d] with M = n_cams*frames*gh*gw,
  * Wt [3d][d], bias [3d]; writes q, k, v [M][d] (heads interleaved by column:
  * head h owns columns h*head_dim ...).  Token row r of chunk `chunk` sits at
- * camera r / (frames*gh*gw), absolute frame chunk*frames + f, grid (h, w). */
+ * camera r / (frames*gh*gw), absolute frame chunk*frames + f, grid (h, w).
+ * head_dim % 16 == 0 for XC_F32; head_dim % 32 == 0 and d % 256 == 0 for
+ * XC_BF16 (XC_EINVAL otherwise, before any launch). */
 xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int chunk,
                          int d, int head_dim, float rope_theta, const void *A,
                          const void *Wt, const float *bias, void *q, void *k, void *v,

@@ -1585,9 +1585,13 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
                          float rope_theta, const void *A, const void *Wt, const float *bias, void *q, void *k,
                          void *v, void *stream) {
     if (n_cams < 1 || frames < 1 || gh < 1 || gw < 1 || chunk < 0 || head_dim < 16 || head_dim % 16 != 0 ||
-        d % head_dim != 0 || A == nullptr || Wt == nullptr || bias == nullptr || q == nullptr || k == nullptr ||
-        v == nullptr)
+        d < head_dim || d % head_dim != 0 || A == nullptr || Wt == nullptr || bias == nullptr || q == nullptr ||
+        k == nullptr || v == nullptr)
         OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: bad argument");
+    if (dtype != XC_BF16 && dtype != XC_F32) OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: dtype");
+    // the bf16 epilogue rotates 32 columns, 16 consecutive pairs of one head, at a time
+    if (dtype == XC_BF16 && (d % 256 != 0 || head_dim % 32 != 0))
+        OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: bf16 needs d %% 256 == 0, head_dim %% 32 == 0");
     // per-call RoPE layout and table (operator path; the chunk step keeps its own)
     static int *axis = nullptr, *off = nullptr;
     static float2 *cs = nullptr;
@@ -1636,18 +1640,15 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
     ep.rope_cs = cs;
     cudaStream_t st = st0;
     if (dtype == XC_BF16) {
-        if ((3 * d) % 256 != 0 || d % 64 != 0) OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: bf16 needs 3d %% 256, d %% 64");
         CUtensorMap ta;
         WeightMaps tb{};
         const int bn = gemm_tc_bn(EPI_QKV_ROPE, M, 3 * d, d);
         if (!make_tmap_bf16(&ta, A, M, d, 128) || !make_weight_maps(&tb, bn, Wt, 3 * (uint64_t)d, d))
             OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: tensor map");
         OP_CK(gemm_tc(EPI_QKV_ROPE, bn, ta, tb, ep, d, nullptr, op_err_word(), st));
-    } else if (dtype == XC_F32) {
+    } else {
         OP_CK(gemm_simt(EPI_QKV_ROPE, ep, reinterpret_cast<const float *>(A), reinterpret_cast<const float *>(Wt), d,
                         nullptr, st));
-    } else {
-        OP_FAIL(XC_EINVAL, "xc_op_qkv_rope: dtype");
     }
     return XC_OK;
 }

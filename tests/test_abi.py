@@ -75,6 +75,17 @@ def test_host_validation_without_gpu(xb):
     assert xb.LIB.xc_op_attention(1, 0, 1, 1, 64, None, None, None, None, None, 0, None) == xb.XC_EINVAL
 
 
+@pytest.mark.parametrize("dtype,d,hd", [(1, 256, 16), (1, 768, 48), (1, 1280, 80),   # 32-column epilogue blocks
+                                        (1, 64, 64), (1, 192, 64),                  # d % 256
+                                        (0, 64, 24), (0, 0, 16), (2, 256, 64)])
+def test_qkv_rope_shapes_are_checked_before_any_launch(xb, dtype, d, hd):
+    """Rejected on the host: no CUDA call is reached (no GPU needed, and the
+    pointers are not looked at)."""
+    p = ctypes.c_void_p(4096)
+    assert xb.LIB.xc_op_qkv_rope(dtype, 1, 1, 4, 4, 0, d, hd, 1e4, p, p, p, p, p, p, None) == xb.XC_EINVAL
+    assert "xc_op_qkv_rope" in xb.last_error(None)
+
+
 def _cfg(xb, **kw):
     base = dict(n_blocks=2, d_model=64, n_heads=4, head_dim=16, d_ffn=256, c_latent=16, action_dim=2,
                 n_cams=3, frames=2, grid_h=4, grid_w=4, kv_window_chunks=2, n_denoise_steps=4, dtype=0,

@@ -76,7 +76,7 @@ def test_linear_tilings(M, N, K, epi):
 
 # 2550 rows, N = 2304: pairs; 1980 rows: wide single tiles
 @pytest.mark.parametrize("gh,gw", [(17, 25), (15, 22)])
-@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("hd", [32, 64, 96, 128])
 def test_qkv_rope_pairs(hd, gh, gw):
     cams, frames, d, chunk = 3, 2, 768, 5
     M, H = cams * frames * gh * gw, d // hd
