@@ -44,7 +44,9 @@ xc_status xc_op_linear(int dtype, int epilogue, int M, int N, int K, const void 
  * head h owns columns h*head_dim ...).  Token row r of chunk `chunk` sits at
  * camera r / (frames*gh*gw), absolute frame chunk*frames + f, grid (h, w).
  * head_dim % 16 == 0 for XC_F32; head_dim % 32 == 0 and d % 256 == 0 for
- * XC_BF16 (XC_EINVAL otherwise, before any launch). */
+ * XC_BF16 (XC_EINVAL otherwise, before any launch).  The RoPE table of a call
+ * is allocated and freed in stream order: calls may overlap on several streams
+ * and threads, and may be captured. */
 xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int chunk,
                          int d, int head_dim, float rope_theta, const void *A,
                          const void *Wt, const float *bias, void *q, void *k, void *v,
