@@ -12,9 +12,10 @@
 //   wide   (BN = 256, WIDE) one CTA per 128 x 256 tile, four ring stages, where
 //          the row count leaves the pairs a ragged last round;
 //   single (BN = 128, 64) one CTA per 128 x BN tile, for GEMMs with too few
-//          256 x 256 tiles to fill the pairs.  With few tiles a k step waits
-//          for the latency of its loads (some 2200 cycles over the ring's
-//          depth): 64-wide tiles put twice the CTAs and eight stages to work.
+//          256 x 256 tiles to fill the pairs.  With few tiles a k step takes
+//          the MMA warp's chain of instructions (some 340 cycles) at either
+//          width: 64-wide tiles spread the epilogue over twice the CTAs (840 x
+//          512 x 512 5.2 us 128 wide, 4.6 64 wide).
 // Persistent: the CTAs (pairs) walk the output tiles in grouped super-rows
 // (tile_at).  Warp roles (320 threads per CTA):
 //   warp 0         : TMA producer, STAGES-deep ring of (A 128x64, B 128x64)
@@ -39,6 +40,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 #include "xc_kernels.cuh"
@@ -302,36 +304,58 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             };
             // start-address field += offset >> 4 (shared addresses < 256 KB: no carry)
             const uint64_t d0 = sdesc_sw128(smem_u32(smem), 16, 1024);
-            int it = 0, local = 0;
-            bool ok = true;
-            for (int item = worker; ok && item < tw.n_items; item += n_workers, ++local) {
-                const int buf = local & 1;
-                const uint32_t use = (uint32_t)(local >> 1);
-                const uint32_t idesc = BN == 256 && item >= tw.n_full ? idesc_bf16(G::BM, 128, false, false)
-                                                                      : idesc_bf16(G::BM, BN, false, false);
-                if (!wait(&acc_empty[buf], (use & 1) ^ 1)) break;
-                tc_fence_after();
-                const uint32_t acc = tmem + buf * BN;
-                for (int kt = 0; kt < KT; ++kt, ++it) {
-                    const int s = it % G::STAGES;
-                    if (!wait(&full[s], (it / G::STAGES) & 1)) {
-                        ok = false;
-                        break;
-                    }
+            // Where few CTAs share the chip this loop's own chain of
+            // instructions bounds a k step, whatever the tile's width and the
+            // ring's depth.  So stage and parity are counted, not divided out of a
+            // step number, and the next stage is looked at before the MMAs of this
+            // one: 128 x 512 x 13824 42.0 -> 35.6 us, 486 x 1024 x 5888 19.8 -> 17.0,
+            // 684 x 2816 x 4928 17.6 -> 15.6.  Not where the data is not there yet
+            // when looked at: wide tiles wait for their 48 KB a step (2356 x 2048 x
+            // 13824 87.8 us without, 89.5 with), and up to five steps are all in
+            // the ring's first turn (7251 x 768 x 128 5.75 and 5.79, 584 x 7168 x
+            // 320 6.34 and 6.40, 447 x 3072 x 384 4.49 and 4.46).  Two loops,
+            // because a test of K inside one cost all of the gain.
+            auto issue_tiles = [&](auto look) {
+                int local = 0, s = 0;
+                uint32_t ph = 0;
+                bool ok = true, ready = false;
+                for (int item = worker; ok && item < tw.n_items; item += n_workers, ++local) {
+                    const int buf = local & 1;
+                    const uint32_t use = (uint32_t)(local >> 1);
+                    const uint32_t idesc = BN == 256 && item >= tw.n_full ? idesc_bf16(G::BM, 128, false, false)
+                                                                          : idesc_bf16(G::BM, BN, false, false);
+                    if (!wait(&acc_empty[buf], (use & 1) ^ 1)) break;
                     tc_fence_after();
-                    const uint64_t da = d0 + (uint64_t)((s * G::STAGE_BYTES) >> 4);
-                    const uint64_t db = da + (uint64_t)(G::A_BYTES >> 4);
+                    const uint32_t acc = tmem + buf * BN;
+                    for (int kt = 0; kt < KT; ++kt) {
+                        if (!ready && !wait(&full[s], ph)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint64_t da = d0 + (uint64_t)((s * G::STAGE_BYTES) >> 4);
+                        const uint64_t db = da + (uint64_t)(G::A_BYTES >> 4);
+                        uint64_t *const used = &empty[s];
+                        if (++s == G::STAGES) {
+                            s = 0;
+                            ph ^= 1;
+                        }
+                        // (on every step: it says whether the next one need not wait)
+                        if constexpr (decltype(look)::value) ready = __all_sync(0xffffffffu, mbar_test(&full[s], ph));
 #pragma unroll
-                    for (int k = 0; k < GEMM_BK / 16; ++k) {
-                        if constexpr (PAIR) tc_mma_pair_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
-                        else tc_mma_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
+                        for (int k = 0; k < GEMM_BK / 16; ++k) {
+                            if constexpr (PAIR) tc_mma_pair_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
+                            else tc_mma_warp(acc, da + 2 * k, db + 2 * k, idesc, (kt | k) != 0 ? 1u : 0u);
+                        }
+                        if constexpr (PAIR) tc_commit_pair_warp(used);
+                        else tc_commit_warp(used);
                     }
-                    if constexpr (PAIR) tc_commit_pair_warp(&empty[s]);
-                    else tc_commit_warp(&empty[s]);
+                    if constexpr (PAIR) tc_commit_pair_warp(&acc_full[buf]);
+                    else tc_commit_warp(&acc_full[buf]);
                 }
-                if constexpr (PAIR) tc_commit_pair_warp(&acc_full[buf]);
-                else tc_commit_warp(&acc_full[buf]);
-            }
+            };
+            if (WIDE || KT <= 5) issue_tiles(std::false_type{});
+            else issue_tiles(std::true_type{});
         }
     } else {
         // ---------------------------------------------------------- epilogue (warps 2..9)
