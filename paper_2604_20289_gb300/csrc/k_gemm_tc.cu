@@ -224,8 +224,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     uint64_t *acc_empty = acc_full + 2;        // [2]
     uint64_t *ld_bar = acc_empty + 2;          // [8][SLOTS] residual operands of an epilogue warp's slot landed
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ld_bar + 8 * EpiRing<EPI, DEEP, WIDE>::SLOTS);
+    // pair: stages that the leader's and the peer's producer loaded, and that
+    // the MMA warp has seen land; each written to both CTAs by its owner
+    int *stages = reinterpret_cast<int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto publish = [&](int i, int v) {
+        if (lane == 0)
+            for (uint32_t r = 0; r < 2; ++r) st_cluster(map_to_cta(stages + i, r), v);
+    };
     const int KT = K / GEMM_BK;
     constexpr bool PAIR = G::PAIR;
     // worker = CTA or CTA pair; rank 0 of a pair leads (issues its MMAs)
@@ -280,18 +287,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     tma_stage_warp(&full[s], bytes, sa, &tmA, m0, sa + G::A_BYTES, tb, n0, kt * GEMM_BK);
             }
         }
-        // Drain: every copy this warp started has landed before exit.  A
-        // pair's leader waits for both CTAs' bytes, and the peer leaves only
-        // after it (the cluster barrier at the end); the peer sees no barrier
-        // of its own, so when one of its waits ran out it gives its last
-        // copies a fixed 10 ms.
-        if (rank == 0) {
+        // Drain: every copy this warp started has landed before exit (pairs: at
+        // the end, from the counts of both).
+        if constexpr (PAIR) {
+            publish(rank, it);
+        } else {
             for (int j = it - G::STAGES < 0 ? 0 : it - G::STAGES; j < it; ++j)
                 mbar_wait(&full[j % G::STAGES], (j / G::STAGES) & 1, err, ERR_WAIT_PRODUCER);
-        } else if (!ok) {
-            const unsigned long long t0 = global_ns();
-            for (unsigned i = 0; i < WAIT_MAX_ITERS && global_ns() - t0 < 10000000ull; ++i) {
-            }
         }
     } else if (warp == 1) {
         // MMA issue: the whole warp runs the loop (converged) and one elected
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             // 320 6.34 and 6.40, 447 x 3072 x 384 4.49 and 4.46).  Two loops,
             // because a test of K inside one cost all of the gain.
             auto issue_tiles = [&](auto look) {
-                int local = 0, s = 0;
+                int local = 0, s = 0, turns = 0;
                 uint32_t ph = 0;
                 bool ok = true, ready = false;
                 for (int item = worker; ok && item < tw.n_items; item += n_workers, ++local) {
@@ -339,6 +341,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                         if (++s == G::STAGES) {
                             s = 0;
                             ph ^= 1;
+                            ++turns;
                         }
                         // (on every step: it says whether the next one need not wait)
                         if constexpr (decltype(look)::value) ready = __all_sync(0xffffffffu, mbar_test(&full[s], ph));
@@ -353,6 +356,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     if constexpr (PAIR) tc_commit_pair_warp(&acc_full[buf]);
                     else tc_commit_warp(&acc_full[buf]);
                 }
+                if constexpr (PAIR) publish(2, turns * G::STAGES + s);
             };
             if (WIDE || KT <= 5) issue_tiles(std::false_type{});
             else issue_tiles(std::true_type{});
@@ -524,7 +528,28 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync_all();           // no MMA, commit or arrival of the pair still to come
+    if constexpr (PAIR) {
+        cluster_sync_all();                           // no MMA, commit or arrival of the pair still to come
+        // Where a wait ran out, stages are left that no MMA has waited for, and
+        // one CTA may have loaded some that the other has not.  The leader makes
+        // up their count, so that their phases complete when the copies in flight
+        // land, and waits for them; the peer leaves after it.
+        const int n0 = stages[0], n1 = stages[1], seen = stages[2];
+        if (n0 != seen || n1 != seen) {
+            if (rank == 0 && threadIdx.x == 0) {
+                for (int j = seen; j < max(n0, n1); ++j) {
+                    const Tile t = tile_at<G::BM, BN>(tw, worker + j / KT * n_workers);
+                    const uint32_t bytes = (uint32_t)G::A_BYTES + (uint32_t)(t.w / 2) * (GEMM_BK * 2);
+                    uint64_t *b = &full[j % G::STAGES];
+                    if (j >= n1) mbar_complete_tx(b, bytes);       // expected of the peer
+                    if (j >= n0) mbar_expect_tx(b, bytes);         // the peer's alone
+                    mbar_wait(b, (j / G::STAGES) & 1, err, ERR_WAIT_PRODUCER);
+                }
+            }
+            __syncthreads();
+            cluster_sync_all();
+        }
+    }
     if (warp == 1) {
         tc_fence_after();
         if constexpr (PAIR) tmem_dealloc_pair(tmem, G::TMEM_COLS);

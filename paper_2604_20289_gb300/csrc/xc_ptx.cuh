@@ -89,6 +89,15 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return r;
 }
+// A word into another CTA's shared memory (shared::cluster address).
+__device__ __forceinline__ void st_cluster(uint32_t a, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+// Counts `bytes` on a barrier of this CTA as if a copy of that size had landed.
+__device__ __forceinline__ void mbar_complete_tx(uint64_t *bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+                 : "memory");
+}
 // Loads from another CTA's shared memory (shared::cluster address).
 __device__ __forceinline__ float2 ld_cluster2(uint32_t a) {
     float2 v;
