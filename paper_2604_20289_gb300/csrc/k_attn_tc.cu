@@ -875,16 +875,6 @@ __global__ void __launch_bounds__(64)
 
 bool make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
-static int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    }
-    return n;
-}
-
 size_t attn_workspace_bytes(int head_dim) {
     const size_t slots = 2 * ((size_t)sm_count() + 1);
     return slots * 256 * ((size_t)head_dim * sizeof(float) + sizeof(float2));
@@ -892,20 +882,15 @@ size_t attn_workspace_bytes(int head_dim) {
 
 template <int HD, int ORDER>
 static cudaError_t attn_attr() {
-    using A = AttnTile<HD>;
-    static bool attr_set = false;
-    if (attr_set) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<HD, ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               A::SMEM_BYTES);
-    attr_set = e == cudaSuccess;
-    return e;
+    static PerDevice done;
+    return allow_smem(done, attn_tc_kernel<HD, ORDER>, AttnTile<HD>::SMEM_BYTES);
 }
 
 // Clusters of `size` attention CTAs (one per SM) that are resident at once.
 template <int HD>
 static int attn_clusters(int size) {
-    static int known[9];                               // 0: not asked yet
-    if (known[size] == 0) {
+    static PerDevice known[9];
+    return known[size].get([size] {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(size * (sm_count() / size)));
         cfg.blockDim = dim3(AttnTile<HD>::THREADS);
@@ -923,9 +908,8 @@ static int attn_clusters(int size) {
             cudaGetLastError();
             n = 0;
         }
-        known[size] = n > 0 ? n : -1;
-    }
-    return known[size];
+        return n > 0 ? n : -1;
+    });
 }
 
 template <int HD, int ORDER>

@@ -25,16 +25,6 @@ cudaError_t expire_wait(int *err, int code, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-static int n_sm_elem() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    }
-    return n;
-}
-
 // ------------------------------------------------------------ patch embed
 // X0[r][c] = round(sum_k z[r][k] * pe_w[k][c] + pe_b[c]), z float32 [L][16].
 // Each lane owns 4 columns for the whole kernel and keeps their 16 x 4 block
@@ -126,7 +116,7 @@ template <typename T>
 cudaError_t patch_embed(const float *z, const float *w, const float *b, T *out, int L, int C, int d, uint8_t *flags,
                         float *metrics, int B, cudaStream_t st) {
     if (C != 16 || d % 16 != 0) return cudaErrorInvalidValue;
-    const int n_sm = n_sm_elem();
+    const int n_sm = sm_count();
     const int n_cb = (d + PE_COLS - 1) / PE_COLS;
     int n_rb = (16 * n_sm + n_cb - 1) / n_cb;          // many short CTAs: no tail wave to speak of
     const int rows = ((L + n_rb - 1) / n_rb + PE_CHUNK - 1) / PE_CHUNK * PE_CHUNK;
@@ -367,7 +357,7 @@ static cudaError_t ln_mod_cta(const T *x, const float *shift, const float *scale
     // 2000 x 5120 15.1 us with one, 16.6 with two) while every SM still gets
     // several CTAs (200 x 4368: 3.4 us with one, 3.6 with two)
     if constexpr (sizeof(T) == 2)
-        if (M >= 4 * n_sm_elem())
+        if (M >= 4 * sm_count())
             return launch_pdl(ln_mod_cta_kernel<T, KMAX, 2>, dim3((M + 1) / 2), dim3(LN_CTA), 0, st, x, shift, scale, out,
                               M, d, eps, skip);
     return launch_pdl(ln_mod_cta_kernel<T, KMAX, 1>, dim3(M), dim3(LN_CTA), 0, st, x, shift, scale, out, M, d, eps, skip);
@@ -378,7 +368,7 @@ cudaError_t ln_mod(const T *x, const float *shift, const float *scale, T *out, i
                    const uint8_t *skip, cudaStream_t st) {
     if (d % 16 != 0) return cudaErrorInvalidValue;
     if (d <= 512) {
-        const int want = (M + 7) / 8, cap = 2 * n_sm_elem();
+        const int want = (M + 7) / 8, cap = 2 * sm_count();
         return launch_pdl(ln_mod_row_kernel<T>, dim3(want < cap ? want : cap), dim3(256), 0, st, x, shift, scale, out, M, d, eps, skip);
     }
     // 16-byte vectors per thread

@@ -514,13 +514,6 @@ template cudaError_t gate_launch<bf16>(const GateArgs &, cudaStream_t);
 template cudaError_t camera_mean_launch<float>(const GateArgs &, cudaStream_t);
 template cudaError_t camera_mean_launch<bf16>(const GateArgs &, cudaStream_t);
 
-static int current_sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
-    return n;
-}
-
 // Checks the arguments of one operator-level gate evaluation (xc_op_gate and
 // xc_op_gate_static take the same ones) and packs them, scratch not bound.
 // Returns XC_OK or XC_EINVAL with the reason in msg.
@@ -619,7 +612,7 @@ extern "C" {
 size_t xc_op_gate_workspace_bytes(int dtype, int n_cams, int tokens_per_cam, int d) {
     (void)dtype;
     if (n_cams < 1 || tokens_per_cam < 1 || d < 64 || d % 64 != 0) return 0;
-    return xc::gate_geometry(n_cams, tokens_per_cam, d, xc::current_sm_count()).total;
+    return xc::gate_geometry(n_cams, tokens_per_cam, d, xc::sm_count()).total;
 }
 
 static_assert(sizeof(xc_gate_cell) == sizeof(xc::GateCell), "gate cell layout");
@@ -636,7 +629,7 @@ xc_status xc_op_gate(int dtype, int n_cams, int tokens_per_cam, int d, const voi
         snprintf(why, sizeof why, "NULL workspace");
         st = XC_EINVAL;
     }
-    const GateGeom gg = xc::gate_geometry(n_cams, tokens_per_cam, d, xc::current_sm_count());
+    const GateGeom gg = xc::gate_geometry(n_cams, tokens_per_cam, d, xc::sm_count());
     if (st == XC_OK && workspace_bytes < gg.total) {
         snprintf(why, sizeof why, "workspace %zu bytes < %zu needed", workspace_bytes, gg.total);
         st = XC_EINVAL;
@@ -672,7 +665,7 @@ xc_status xc_op_gate_static(int dtype, int n_cams, int tokens_per_cam, int d, co
         xc::set_global_error(msg);
         return st;
     }
-    const GateGeom gg = xc::gate_geometry(n_cams, tokens_per_cam, d, xc::current_sm_count());
+    const GateGeom gg = xc::gate_geometry(n_cams, tokens_per_cam, d, xc::sm_count());
     if (gg.total > xc::GATE_STATIC_SCRATCH_BYTES) {
         snprintf(msg, sizeof msg,
                  "xc_op_gate_static: this geometry needs %zu bytes of scratch, more than the %zu-byte "

@@ -564,7 +564,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapFloatOOBfill);
 
 static EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
+    static std::atomic<EncodeTiledFn> known{nullptr};
+    EncodeTiledFn fn = known.load(std::memory_order_relaxed);
     if (fn == nullptr) {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -572,6 +573,7 @@ static EncodeTiledFn encode_fn() {
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
             fn = reinterpret_cast<EncodeTiledFn>(p);
+        known.store(fn, std::memory_order_relaxed);
     }
     return fn;
 }
@@ -658,24 +660,14 @@ static bool build_epi_maps(EpiMaps &em, const EpiParams &ep) {
     }
 }
 
-static int gemm_sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    }
-    return n;
-}
-
 // CTA pairs resident at once (both CTAs of a pair sit on neighbouring SMs).
 template <int EPI, bool DEEP>
 static int pair_count() {
-    static int n = 0;
-    if (n == 0) {
+    static PerDevice known;
+    return known.get([] {
         using G = GemmTile<256, EPI, DEEP, false>;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2 * (gemm_sm_count() / 2));
+        cfg.gridDim = dim3(2 * (sm_count() / 2));
         cfg.blockDim = dim3(GEMM_THREADS);
         cfg.dynamicSmemBytes = G::SMEM_BYTES;
         cudaLaunchAttribute attr[1];
@@ -688,11 +680,10 @@ static int pair_count() {
         int k = 0;
         if (cudaOccupancyMaxActiveClusters(&k, gemm_tc_kernel<256, EPI, DEEP, false>, &cfg) != cudaSuccess || k < 1) {
             cudaGetLastError();
-            k = gemm_sm_count() / 2;
+            k = sm_count() / 2;
         }
-        n = k < 1 ? 1 : k;
-    }
-    return n;
+        return k < 1 ? 1 : k;
+    });
 }
 
 // Walk of a pair grid over 256 x 256 tiles: a remainder of at most half of
@@ -723,7 +714,7 @@ static TileWalk pair_walk(int M, int N, int workers) {
 // 33.2 / 24.0 / 27.1, x 1024 16.6 / 13.3 / 12.6, 7200 x 2560 x 1024 40.5 / 43.7 /
 // 48.7; 239 x 12032 x 3712 22.0 / - / 27.7.
 int gemm_tc_bn(int epi, int M, int N, int K) {
-    const long n_sm = gemm_sm_count(), pairs = n_sm / 2 < 1 ? 1 : n_sm / 2;
+    const long n_sm = sm_count(), pairs = n_sm / 2 < 1 ? 1 : n_sm / 2;
     const long tm = (M + 127) / 128, t128 = tm * (N / 128), r128 = (t128 + n_sm - 1) / n_sm;
     if (2 * t128 <= n_sm) return 64;
     if (N % 256 != 0) return 128;
@@ -749,13 +740,10 @@ static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const 
     auto kern = gemm_tc_kernel<BN, EPI, DEEP, WIDE>;
     EpiMaps em;
     if (!build_epi_maps<EPI>(em, ep)) return cudaErrorInvalidValue;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    int workers = gemm_sm_count();
+    static PerDevice smem_done;
+    const cudaError_t e = allow_smem(smem_done, kern, G::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    int workers = sm_count();
     TileWalk tw;
     if constexpr (G::PAIR) {
         workers = pair_count<EPI, DEEP>();

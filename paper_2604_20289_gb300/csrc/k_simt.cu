@@ -157,16 +157,6 @@ __global__ void __launch_bounds__(SG_THREADS)
     }
 }
 
-static int simt_sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    }
-    return n;
-}
-
 template <int EPI, bool VEC>
 static cudaError_t gemm_simt_vec(const EpiParams &ep, const float *A, const float *Wt, int K, const uint8_t *skip,
                                  cudaStream_t st) {
@@ -176,7 +166,7 @@ static cudaError_t gemm_simt_vec(const EpiParams &ep, const float *A, const floa
     // 12.9 against 12.8, 128 tiles (1024 x 512 x 512) 24.4 against 49.6; the
     // line is at 3/8 of the SMs
     const long tiles = (long)((ep.M + SG_TILE - 1) / SG_TILE) * ((ep.N + SG_TILE - 1) / SG_TILE);
-    if (8 * tiles >= 3L * simt_sm_count())
+    if (8 * tiles >= 3L * sm_count())
         return launch_pdl(gemm_simt_tile<EPI, VEC>, dim3((unsigned)tiles), dim3(SG_THREADS), 0, st, ep, A, Wt, K, skip);
     return launch_pdl(gemm_simt_small<EPI, VEC>, dim3((unsigned)((ep.M + 15) / 16 * (ep.N / 16))), dim3(SG_THREADS), 0,
                       st, ep, A, Wt, K, skip);
@@ -366,7 +356,7 @@ static cudaError_t attn_simt_vec(const float *q, const float *k, const float *v,
     // registers: one CTA per SM at hd 64, two below), four beyond.  Both
     // measured, eight / four warps: 300 x 2000 x 4 x 32 (76 CTAs) 53 / 91
     // us, 1024 x 3072 x 2 x 64 (128) 115 / 183, 640 x 640 x 4 x 64 (160) 57 / 50
-    if (n > (HD >= 64 ? 1L : 2L) * simt_sm_count())
+    if (n > (HD >= 64 ? 1L : 2L) * sm_count())
         return launch_pdl(attn_simt_f32<HD, 4, VEC>, dim3((unsigned)n), dim3(128), 0, st, q, k, v, o, Lq, n_keys, H, skip);
     return launch_pdl(attn_simt_f32<HD, 8, VEC>, dim3((unsigned)n), dim3(256), 0, st, q, k, v, o, Lq, n_keys, H, skip);
 }

@@ -1513,10 +1513,17 @@ xc_status xc_chunk_step(xc_ctx *ctx, const float *latent, const float *action, f
 }
 
 // ---------------------------------------------------------------- op entries
+// Error word of the operator entry points on the current device, made by the
+// first call on it.
 static int *op_err_word() {
-    static int *p = nullptr;
+    static std::mutex mu;
+    static std::map<int, int *> words;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    int *&p = words[dev];
     if (p == nullptr) {
-        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) return nullptr;
+        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) return p = nullptr;
         cudaMemset(p, 0, sizeof(int));
     }
     return p;
@@ -1753,9 +1760,7 @@ xc_status xc_op_residual_reuse(int dtype, long n, const void *x, const void *rha
     if (n < 0 || n % 16 != 0 || x == nullptr || rhat == nullptr || out == nullptr)
         OP_FAIL(XC_EINVAL, "xc_op_residual_reuse: bad argument (n %% 16 == 0 required)");
     if (n == 0) return XC_OK;
-    int dev = 0, n_sm = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const int n_sm = sm_count();
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (dtype == XC_BF16)
         OP_CK(residual_reuse<bf16>(reinterpret_cast<const bf16 *>(x), reinterpret_cast<const bf16 *>(rhat),

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/xcache.h"
 #include "../../include/xcache_ops.h"
 
@@ -43,6 +45,47 @@ template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args &&...args) {
     return launch_pdl_cluster(kernel, 1, grid, block, smem, st, static_cast<Args &&>(args)...);
+}
+
+// A value that a launch needs and that is asked for once per device (an answer
+// of 0 is not kept).  Threads that ask at the same time get the same.
+struct PerDevice {
+    static constexpr int MAX = 64;
+    std::atomic<int> known[MAX] = {};
+    template <typename Ask>
+    int get(Ask ask) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX) return ask();
+        int v = known[dev].load(std::memory_order_relaxed);
+        if (v == 0) {
+            v = ask();
+            known[dev].store(v, std::memory_order_relaxed);
+        }
+        return v;
+    }
+};
+// SMs of the current device (1 where it cannot be asked).
+inline int sm_count() {
+    static PerDevice sms;
+    const int n = sms.get([] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            v = 0;
+        return v;
+    });
+    return n < 1 ? 1 : n;
+}
+// Lets a kernel have `bytes` of dynamic shared memory, once per device and
+// kernel (`done` is that kernel's).
+template <typename Kernel>
+inline cudaError_t allow_smem(PerDevice &done, Kernel kern, int bytes) {
+    cudaError_t e = cudaSuccess;
+    done.get([&] {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        return e == cudaSuccess ? 1 : 0;
+    });
+    return e;
 }
 
 typedef __nv_bfloat16 bf16;
