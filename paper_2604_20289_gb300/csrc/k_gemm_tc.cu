@@ -95,6 +95,7 @@ struct GemmTile {
     static constexpr int EPI_WARPS = PAIR ? 16 : 8;    // that release an accumulator
     static_assert(STAGES >= 3, "main-loop ring too shallow");
     static_assert(SMEM_BYTES <= GEMM_SMEM_LIMIT, "shared memory");
+    static_assert(!PAIR || 2 * SMEM_BYTES > GEMM_SMEM_LIMIT, "one pair CTA per SM (pair_count)");
 };
 
 // Tensor maps of the epilogue (32 x 32 bf16 boxes, 64-byte swizzle):
@@ -665,12 +666,15 @@ static bool build_epi_maps(EpiMaps &em, const EpiParams &ep) {
     }
 }
 
-// CTA pairs resident at once (both CTAs of a pair sit on neighbouring SMs).
-template <int EPI, bool DEEP>
+// CTA pairs resident at once (both CTAs of a pair sit on neighbouring SMs); the
+// same for every pair kernel, whose shared memory leaves room for one CTA on an
+// SM.  The tiling rule and the launch walk with the same count.
 static int pair_count() {
     static PerDevice known;
     return known.get([] {
-        using G = GemmTile<256, EPI, DEEP, false>;
+        using G = GemmTile<256, EPI_BIAS, false, false>;
+        auto kern = gemm_tc_kernel<256, EPI_BIAS, false, false>;
+        static PerDevice smem_done;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2 * (sm_count() / 2));
         cfg.blockDim = dim3(GEMM_THREADS);
@@ -683,7 +687,8 @@ static int pair_count() {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int k = 0;
-        if (cudaOccupancyMaxActiveClusters(&k, gemm_tc_kernel<256, EPI, DEEP, false>, &cfg) != cudaSuccess || k < 1) {
+        if (allow_smem(smem_done, kern, G::SMEM_BYTES) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&k, kern, &cfg) != cudaSuccess || k < 1) {
             cudaGetLastError();
             k = sm_count() / 2;
         }
@@ -719,7 +724,7 @@ static TileWalk pair_walk(int M, int N, int workers) {
 // 33.2 / 24.0 / 27.1, x 1024 16.6 / 13.3 / 12.6, 7200 x 2560 x 1024 40.5 / 43.7 /
 // 48.7; 239 x 12032 x 3712 22.0 / - / 27.7.
 int gemm_tc_bn(int epi, int M, int N, int K) {
-    const long n_sm = sm_count(), pairs = n_sm / 2 < 1 ? 1 : n_sm / 2;
+    const long n_sm = sm_count(), pairs = pair_count();
     const long tm = (M + 127) / 128, t128 = tm * (N / 128), r128 = (t128 + n_sm - 1) / n_sm;
     if (2 * t128 <= n_sm) return 64;
     if (N % 256 != 0) return 128;
@@ -751,7 +756,7 @@ static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const 
     int workers = sm_count();
     TileWalk tw;
     if constexpr (G::PAIR) {
-        workers = pair_count<EPI, DEEP>();
+        workers = pair_count();
         tw = pair_walk(ep.M, ep.N, workers);
     } else {
         tw.tiles_m = (ep.M + GEMM_BM - 1) / GEMM_BM;
