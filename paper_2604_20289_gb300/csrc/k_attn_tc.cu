@@ -938,48 +938,54 @@ static cudaError_t launch_attn_(const CUtensorMap &tq, const CUtensorMap &tk, co
     return e;
 }
 
+// What a launch runs: an order, its split, the CTAs of a cluster and what the
+// merge launch has to merge (0: no such launch).
+struct AttnPlan {
+    int order, cluster, n_combine;
+    AttnSplit sp;
+};
+
 // Work order (see AttnSplit).  Cutting units balances the SMs at the price of
-// partials and their merge, CUT key tiles' time or so.
-//  * Whole units in waves where the longest CTA has at most CUT key tiles
-//    more than an even share (cross-attention to a few hundred condition
-//    tokens: 12960 x 300 x 12 heads of 128 60.8 us cut, 37.1 whole), and
-//    without a workspace.
+// partials and their merge.  Both sides are compared in key tiles (1.2 us at hd
+// 64, 1.6 at hd 128): whole units take the longest CTA's tiles, a cut the tiles
+// of a CTA's share and the time of its merge, fitted to 450 shapes measured both
+// ways (98 to 12960 queries, 3 to 48 key tiles, 2 to 2040 units; the choice
+// costs at most 3 % of the better one).
 //  * Fewer units than SMs: every unit is split over the same number of CTAs,
-//    so that no CTA touches two units; more than half as many units as SMs,
-//    over all SMs.  One CTA per unit before: 840 x 2520 x 4 heads of 64 26.6
-//    -> 16.2 us (14.3 in clusters), 1000 x 10000 x 2 heads of 128 118 -> 28.
+//    so that no CTA touches two units: in clusters, which merge in rounds of 8
+//    warps per CTA over the unit's 16-row blocks and read a partial of every
+//    CTA in each (200 x 590 x 12 heads of 64: 10.1 us whole, 12.4 in clusters of
+//    3; 98 x 974 x 12 13.2 whole, 10.5 in clusters of 4), or merged through
+//    global memory (1000 x 718 x 12 of 128 14.6 whole, 16.0 by 3; 300 x 974 x 6
+//    17.1 whole, 14.6 by 4; 1000 x 10000 x 2 118 and 27).
+//  * More than half as many units as SMs: over all SMs, a CTA touching two
+//    units (512 x 1614 x 40 of 64 19.5 whole, 20.9 cut; 512 x 2510 x 40 27.3 and
+//    25.3; 1000 x 2560 x 24 of 128 34.6 and 37.3, 512 x 3278 x 40 43.4 and 38.2).
 //  * Waves with the remaining units split when there are many waves (W >= 8)
 //    and the K / V of all heads exceed L2 -- measured at the 14B shape (40
 //    heads x 20 MB of K / V, W = 13): 40.7 -> 1.2 GB of DRAM traffic per
 //    launch at the same attention time, the GPU's power then allowing a
 //    higher clock under its cap (1500 -> 1965 MHz, 0.766 -> 0.801 chunks/s).
-//  * Else contiguous shares; at the 1.3B shape (W = 4) the waves were 4 %
-//    slower per launch.
+//  * Else contiguous shares (at the 1.3B shape, W = 4, the waves were 4 %
+//    slower per launch): 4000 x 718 x 12 of 64 20.3 whole, 21.5 cut; 4000 x 1230 x
+//    12 29.2 and 27.0; 12960 x 718 x 12 of 128 56.9 and 60.8, 4000 x 1408 x 12 39.6
+//    and 37.5.
 template <int HD>
-static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
-                               const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws,
-                               size_t ws_bytes, const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {
+static AttnPlan attn_plan(int Lq, int n_keys, int n_heads, bool can_cut) {
     using A = AttnTile<HD>;
-    constexpr int CUT = 5;
-    AttnSplit sp;
+    AttnPlan pl{ORDER_WAVE, 1, 0, {}};
+    AttnSplit &sp = pl.sp;
     sp.n_kt = (n_keys + A::BKV - 1) / A::BKV;
     sp.n_qblk = (Lq + A::QT * A::BQ - 1) / (A::QT * A::BQ);
     const int n_units = sp.n_qblk * n_heads;
     const int n_sm = sm_count();
-    // (partials leave by bulk copies: 16-byte aligned)
-    const bool can_cut = ws != nullptr && ws_bytes >= attn_workspace_bytes(HD) &&
-                         (reinterpret_cast<uintptr_t>(ws) & 15) == 0;
     sp.T = (long long)n_units * sp.n_kt;
     sp.T2 = 0;
     sp.G = n_units < n_sm ? n_units : n_sm;
     sp.W = n_units / sp.G;
     sp.R = n_units - sp.W * sp.G;
-    const long long longest = (long long)(sp.W + (sp.R > 0 ? 1 : 0)) * sp.n_kt;
-    // a unit of one query tile at hd 128 walks its keys faster: 98 x 717 x 19
-    // heads (6 key tiles) 13.6 us whole, 14.5 cut; 264 x 736 x 6 16.0 and 14.3
-    const int cut = HD == 128 && Lq <= A::BQ ? CUT + 1 : CUT;
-    if (!can_cut || (longest - cut) * n_sm <= sp.T)
-        return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, 0, ws, skip, err, n_launched, st);
+    const double whole = (double)(sp.W + (sp.R > 0 ? 1 : 0)) * sp.n_kt, even = (double)sp.T / n_sm;
+    if (!can_cut || whole <= even) return pl;
     if (n_units < n_sm) {
         // One cluster of up to 8 CTAs per unit, as many as can all be resident
         // at once, while a CTA has at most 8 key tiles: beyond, more CTAs per
@@ -990,40 +996,65 @@ static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, con
         // (clusters of 6) 20.4 -> 19.5; at hd 64 by 10 heads 18.8 -> 18.4, 6
         // heads 17.4 -> 14.6, 4 heads 16.4 -> 14.3.
         constexpr int CL_MIN = HD == 64 ? 2 : 6;
-        int cl = std::min(8, std::min(n_sm / n_units, (sp.n_kt + 1) / 2));
+        const int most = std::min(n_sm / n_units, (sp.n_kt + 1) / 2);    // CTAs of a unit, each two tiles
+        int cl = std::min(8, most);
         while (cl >= CL_MIN && n_units > attn_clusters<HD>(cl)) --cl;
-        if (cl >= CL_MIN && sp.n_kt <= 8 * cl) {
-            sp.G = n_units * cl;
-            sp.W = sp.R = 0;
-            sp.T2 = sp.T;
-            return launch_attn_<HD, ORDER_CLUSTER>(tq, tk, tv, to, o, Lq, n_keys, d, sp, cl, 0, ws, skip, err,
-                                                   n_launched, st);
-        }
-        // CTAs per unit: a key tile takes a CTA about 1.2 us and a partial the
-        // merge about 0.4, so some sqrt(3 n_kt) of them are best (300 x 30000
-        // x 1 head of 128: 76 / 59 / 40 per unit 66 / 53 / 43 us; 474 x 8116 x
-        // 2 heads of 64: 32 / 16 / 11 30 / 21.8 / 21.3)
+        // CTAs per unit otherwise: a key tile takes a CTA about 1.2 us and a
+        // partial the merge about 0.4, so some sqrt(3 n_kt) of them are best (300
+        // x 30000 x 1 head of 128: 76 / 59 / 40 per unit 66 / 53 / 43 us; 474 x
+        // 8116 x 2 heads of 64: 32 / 16 / 11 30 / 21.8 / 21.3)
         int per = 1;
         while (per * per < 3 * sp.n_kt) ++per;
-        per = std::min(per, std::min(n_sm / n_units, (sp.n_kt + 1) / 2));
-        // over all SMs, two pieces per CTA, costs hd 64 some 7 key tiles (899 x
-        // 3493 x 30 heads, 28 key tiles on 120 SMs or 22.1 on all: 36.6 us
-        // whole, 37.9 cut; 993 x 2949 x 35 of 128 43.1 whole, 41.5 cut)
-        if (HD == 64 && per < 2 && (sp.n_kt - 7) * n_sm <= sp.T)
-            return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, 0, ws, skip, err, n_launched, st);
-        sp.G = per >= 2 ? n_units * per : n_sm;
+        per = std::min(per, most);
+        double cut;
+        if (cl >= CL_MIN && sp.n_kt <= 8 * cl) {
+            const int blocks = (std::min(Lq, A::QT * A::BQ) + 15) / 16 * (HD / 32), rounds = (blocks + 8 * cl - 1) / (8 * cl);
+            cut = (sp.n_kt + cl - 1) / cl + (HD == 64 ? 2.5 + 0.4 * rounds * cl : 3.4 + 0.27 * rounds * cl);
+            pl.order = ORDER_CLUSTER;
+            pl.cluster = cl;
+        } else if (per >= 2) {
+            cut = (sp.n_kt + per - 1) / per + 2.8 + 0.4 * per + 0.02 * n_units;
+        } else {
+            cut = even + (HD == 64 ? 8.0 : 10.5);
+        }
+        if (whole <= cut) {
+            pl.order = ORDER_WAVE;
+            pl.cluster = 1;
+            return pl;
+        }
+        sp.G = pl.order == ORDER_CLUSTER ? n_units * cl : per >= 2 ? n_units * per : n_sm;
         sp.W = sp.R = 0;
         sp.T2 = sp.T;
-        return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, n_units, ws, skip, err, n_launched, st);
+        pl.n_combine = pl.order == ORDER_CLUSTER ? 0 : n_units;
+        return pl;
     }
-    const double kv_bytes = 2.0 * n_keys * (double)d * sizeof(bf16);
+    if (whole <= even + (HD == 64 ? 5.0 : 7.0)) return pl;
+    const double kv_bytes = 2.0 * n_keys * (double)(n_heads * HD) * sizeof(bf16);
     if (sp.W >= 8 && kv_bytes > 128.0 * 1024 * 1024) {
-        const int n_rem = sp.R;
-        sp.T2 = (long long)n_rem * sp.n_kt;
+        pl.n_combine = sp.R;
+        sp.T2 = (long long)sp.R * sp.n_kt;
         sp.R = 0;
-        return launch_attn_<HD, ORDER_WAVE>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, n_rem, ws, skip, err, n_launched, st);
+        return pl;
     }
-    return launch_attn_<HD, ORDER_CONTIGUOUS>(tq, tk, tv, to, o, Lq, n_keys, d, sp, 1, sp.G - 1, ws, skip, err, n_launched, st);
+    pl.order = ORDER_CONTIGUOUS;
+    pl.n_combine = sp.G - 1;
+    return pl;
+}
+
+template <int HD>
+static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
+                               const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws,
+                               size_t ws_bytes, const uint8_t *skip, int *err, int *n_launched, cudaStream_t st) {
+    // (partials leave by bulk copies: 16-byte aligned)
+    const bool can_cut = ws != nullptr && ws_bytes >= attn_workspace_bytes(HD) &&
+                         (reinterpret_cast<uintptr_t>(ws) & 15) == 0;
+    const AttnPlan pl = attn_plan<HD>(Lq, n_keys, n_heads, can_cut);
+    auto run = [&](auto launch) {
+        return launch(tq, tk, tv, to, o, Lq, n_keys, d, pl.sp, pl.cluster, pl.n_combine, ws, skip, err, n_launched, st);
+    };
+    if (pl.order == ORDER_CLUSTER) return run(launch_attn_<HD, ORDER_CLUSTER>);
+    if (pl.order == ORDER_CONTIGUOUS) return run(launch_attn_<HD, ORDER_CONTIGUOUS>);
+    return run(launch_attn_<HD, ORDER_WAVE>);
 }
 
 // q [Lq][d], k / v maps over [>= n_keys][d] (boxes of 128 rows), o [Lq][d] and
