@@ -156,6 +156,20 @@ xc_status xc_op_gate_static(int dtype, int n_cams, int tokens_per_cam, int d, co
  * (synchronising).  0 = no error. */
 int xc_op_device_error(void);
 
+/* ---- testing hooks (no counterpart in the paper) ----
+ * What the dispatch rules choose on the current device, for tests that are
+ * to reach a certain kernel; nothing is launched.
+ * xc_debug_gemm_tiling: tiling of a bf16 GEMM (epilogue: an xc_epilogue, or 16
+ * for xc_op_qkv_rope with N = 3 d): columns of a tile by one CTA, 64, 128 or
+ * 257 (256 columns); 256 for CTA pairs.  tiles: full tiles and half tiles.
+ * xc_debug_attention_plan: order of a bf16 attention: 0 contiguous shares, 1
+ * waves (whole units, the remaining ones split), 2 clusters.  plan: CTAs, CTAs
+ * of a cluster, units or boundaries that a second launch merges, whole units
+ * per CTA.  Both: 0 / -1 for a shape that the entry point refuses. */
+int xc_debug_gemm_tiling(int epilogue, int M, int N, int K, int tiles[2]);
+int xc_debug_attention_plan(int Lq, int n_keys, int n_heads, int head_dim, int with_workspace,
+                            int plan[4]);
+
 #ifdef __cplusplus
 }
 #endif

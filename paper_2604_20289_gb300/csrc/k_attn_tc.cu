@@ -1058,6 +1058,16 @@ static cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, con
     return run(launch_attn_<HD, ORDER_WAVE>);
 }
 
+int attn_tc_plan(int head_dim, int Lq, int n_keys, int n_heads, bool can_cut, int plan[4]) {
+    const AttnPlan pl = head_dim == 64 ? attn_plan<64>(Lq, n_keys, n_heads, can_cut)
+                                       : attn_plan<128>(Lq, n_keys, n_heads, can_cut);
+    plan[0] = pl.sp.G;
+    plan[1] = pl.cluster;
+    plan[2] = pl.n_combine;
+    plan[3] = pl.sp.W;
+    return pl.order;
+}
+
 // q [Lq][d], k / v maps over [>= n_keys][d] (boxes of 128 rows), o [Lq][d] and
 // its map (boxes of 32 rows); hd in {64, 128}.  ws: attn_workspace_bytes(hd)
 // bytes, 16-byte aligned, let units be cut between CTAs (nullptr, smaller or

@@ -743,6 +743,20 @@ int gemm_tc_bn(int epi, int M, int N, int K) {
     return pair <= narrow ? 256 : 128;
 }
 
+static TileWalk tile_walk(int bn, int M, int N) {
+    if (bn == 256) return pair_walk(M, N, pair_count());
+    TileWalk tw;
+    tw.tiles_m = (M + GEMM_BM - 1) / GEMM_BM;
+    tw.tiles_n = N / (bn == GEMM_WIDE ? 256 : bn);
+    tw.n_full = tw.n_items = tw.tiles_m * tw.tiles_n;
+    return tw;
+}
+void gemm_tc_tiles(int bn, int M, int N, int *full, int *half) {
+    const TileWalk tw = tile_walk(bn, M, N);
+    *full = tw.n_full;
+    *half = tw.n_items - tw.n_full;
+}
+
 template <int EPI, int BN, bool DEEP = false, bool WIDE = false>
 static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                              const uint8_t *skip, int *err, cudaStream_t st) {
@@ -753,16 +767,8 @@ static cudaError_t launch_tc(const CUtensorMap &ta, const WeightMaps &tb, const 
     static PerDevice smem_done;
     const cudaError_t e = allow_smem(smem_done, kern, G::SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    int workers = sm_count();
-    TileWalk tw;
-    if constexpr (G::PAIR) {
-        workers = pair_count();
-        tw = pair_walk(ep.M, ep.N, workers);
-    } else {
-        tw.tiles_m = (ep.M + GEMM_BM - 1) / GEMM_BM;
-        tw.tiles_n = ep.N / BN;
-        tw.n_full = tw.n_items = tw.tiles_m * tw.tiles_n;
-    }
+    int workers = G::PAIR ? pair_count() : sm_count();
+    const TileWalk tw = tile_walk(WIDE ? GEMM_WIDE : BN, ep.M, ep.N);
     if (tw.n_items < workers) workers = tw.n_items;
     return launch_pdl_cluster(kern, G::PAIR ? 2 : 1, dim3(G::PAIR ? 2 * workers : workers), dim3(GEMM_THREADS), G::SMEM_BYTES, st,
                               ta, tb, em, ep, K, tw, skip, err);

@@ -1773,4 +1773,17 @@ xc_status xc_op_residual_reuse(int dtype, long n, const void *x, const void *rha
     return XC_OK;
 }
 
+int xc_debug_gemm_tiling(int epilogue, int M, int N, int K, int tiles[2]) {
+    const bool known = (epilogue >= XC_EPI_BIAS && epilogue <= XC_EPI_RESID_CACHE) || epilogue == EPI_QKV_ROPE;
+    if (!known || M < 1 || N < 256 || N % 256 != 0 || K < 64 || K % 64 != 0 || tiles == nullptr) return 0;
+    const int bn = gemm_tc_bn(epilogue, M, N, K);
+    gemm_tc_tiles(bn, M, N, &tiles[0], &tiles[1]);
+    return bn;
+}
+
+int xc_debug_attention_plan(int Lq, int n_keys, int n_heads, int head_dim, int with_workspace, int plan[4]) {
+    if (Lq < 1 || n_keys < 1 || n_heads < 1 || (head_dim != 64 && head_dim != 128) || plan == nullptr) return -1;
+    return attn_tc_plan(head_dim, Lq, n_keys, n_heads, with_workspace != 0, plan);
+}
+
 }  // extern "C"

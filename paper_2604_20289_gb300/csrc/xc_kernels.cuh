@@ -103,12 +103,14 @@ inline bool make_weight_maps(WeightMaps *m, int bn, const void *base, uint64_t N
            (!(all || bn == GEMM_WIDE) || make_tmap_bf16(&m->box256, base, N, K, 256));
 }
 int gemm_tc_bn(int epi, int M, int N, int K);
+void gemm_tc_tiles(int bn, int M, int N, int *full, int *half);    // of that tiling
 cudaError_t gemm_tc(int epi, int bn, const CUtensorMap &ta, const WeightMaps &tb, const EpiParams &ep, int K,
                     const uint8_t *skip, int *err, cudaStream_t st);
 cudaError_t attn_tc(int head_dim, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv,
                     const CUtensorMap &to, bf16 *o, int Lq, int n_keys, int n_heads, int d, void *ws, size_t ws_bytes, const uint8_t *skip, int *err,
                     int *n_launched, cudaStream_t st);
 size_t attn_workspace_bytes(int head_dim);
+int attn_tc_plan(int head_dim, int Lq, int n_keys, int n_heads, bool can_cut, int plan[4]);   // see xc_debug_attention_plan
 cudaError_t gemm_simt(int epi, const EpiParams &ep, const float *A, const float *Wt, int K, const uint8_t *skip,
                       cudaStream_t st);
 cudaError_t attn_simt(int head_dim, const float *q, const float *k, const float *v, float *o, int Lq, int n_keys,

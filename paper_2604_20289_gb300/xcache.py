@@ -116,6 +116,8 @@ SIGNATURES = {
                         _P, _P, _P, _P, _P, ctypes.c_size_t, _P]),
     "xc_op_gate_static": (_I, [_I, _I, _I, _I, _P, _P, _I, _P, _P, _P, _P, _I, _I, _I,
                                ctypes.POINTER(GateParams), _P, _P, _P, _P, _P]),
+    "xc_debug_gemm_tiling": (_I, [_I, _I, _I, _I, ctypes.POINTER(_I)]),
+    "xc_debug_attention_plan": (_I, [_I, _I, _I, _I, _I, ctypes.POINTER(_I)]),
 }
 
 
@@ -344,6 +346,19 @@ def op_residual_reuse(dtype, x, rhat, out, stream=None):
 
 def op_device_error() -> int:
     return LIB.xc_op_device_error()
+
+
+def debug_gemm_tiling(epilogue, M, N, K):
+    """(tiling, full tiles, half tiles) of a bf16 GEMM on the current device."""
+    tiles = (ctypes.c_int * 2)()
+    return (LIB.xc_debug_gemm_tiling(epilogue, M, N, K, tiles), *tiles)
+
+
+def debug_attention_plan(Lq, n_keys, n_heads, head_dim, with_workspace=True):
+    """(order, CTAs, CTAs of a cluster, merged units or boundaries, whole units
+    per CTA) of a bf16 attention on the current device."""
+    plan = (ctypes.c_int * 4)()
+    return (LIB.xc_debug_attention_plan(Lq, n_keys, n_heads, head_dim, int(with_workspace), plan), *plan)
 
 
 class GateCell(ctypes.Structure):

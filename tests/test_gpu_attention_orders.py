@@ -1,7 +1,9 @@
 """bf16 attention's work orders at the sizes where they can go wrong: units
 split over several CTAs (evenly, and over all SMs with shares that touch two
-units), whole units in waves with and without a last round, no workspace, a
-second query tile without a row, ragged keys, one key tile; scores that
+units), whole units in waves with and without a last round, waves whose
+remaining units give some CTAs nothing, no workspace, a second query tile
+without a row, ragged keys, one key tile (the order that a case is for is
+asserted); scores that
 outgrow the running max at head_dim 128, whose later tiles take no max of
 their own; and scores of a later tile that are not finite.
 
@@ -40,20 +42,64 @@ def check(q, k, v, H, hd, workspace):
     assert xb.op_device_error() == 0
 
 
-# (Lq, Lk, H, hd) on 152 SMs: 16 units in clusters; one unit in a cluster of 8;
-# 90 units over all SMs (shares touch two units); 2 units of 3 tiles; whole
-# units: 4 of them, 160 (a second round of 8), 240; contiguous cut: 189 units;
-# clusters of 3, of 6 at hd 128; 4 units split 15 ways
-@pytest.mark.parametrize("Lq,Lk,H,hd", [(840, 2520, 4, 64), (130, 5000, 1, 128), (2196, 3000, 10, 64),
-                                        (300, 300, 1, 128), (100, 77, 4, 64), (2500, 500, 16, 128),
-                                        (5000, 129, 12, 64), (2100, 2600, 21, 64),
-                                        (1400, 1000, 7, 64), (840, 2520, 6, 128), (300, 9000, 2, 128)])
+SMS = torch.cuda.get_device_properties(0).multi_processor_count
+CONTIGUOUS, WAVE, CLUSTER = 0, 1, 2
+# (Lq, Lk, H, hd, (order, merged) with a workspace on 152 SMs): merged = units or
+# boundaries that the second launch merges
+ORDERS = [
+    (840, 2520, 4, 64, (CLUSTER, 0)),            # 16 units in clusters of 8
+    (130, 5000, 1, 128, (CLUSTER, 0)),           # one unit
+    (1400, 1000, 7, 64, (CLUSTER, 0)),           # 42 units in clusters of 3
+    (600, 1450, 2, 128, (CLUSTER, 0)),           # 6 in clusters of 6
+    (840, 2520, 6, 128, None),                   # 24 in clusters of 6 where so many fit, else split 6 ways
+    (300, 9000, 2, 128, (WAVE, 4)),              # 4 units split 15 ways
+    (2196, 3000, 10, 64, (WAVE, 90)),            # 90 units over all SMs: shares touch two units
+    (512, 3000, 40, 128, (WAVE, 80)),
+    (300, 300, 1, 128, (CONTIGUOUS, 0)),         # whole: 2 units of 3 tiles
+    (100, 77, 4, 64, (CONTIGUOUS, 0)),
+    (2500, 500, 16, 128, (WAVE, 0)),             # whole: 160, a second round of 8
+    (5000, 129, 12, 64, (WAVE, 0)),
+    (2100, 2600, 21, 64, (CONTIGUOUS, 151)),     # 189 units, cut at the CTAs' boundaries
+    (1000, 1100, 40, 128, (CONTIGUOUS, 151)),
+]
+
+
+@pytest.mark.parametrize("Lq,Lk,H,hd,plan", ORDERS)
 @pytest.mark.parametrize("workspace", ["auto", None])
-def test_attention_orders(Lq, Lk, H, hd, workspace):
+def test_attention_orders(Lq, Lk, H, hd, plan, workspace):
     d = H * hd
+    got = xb.debug_attention_plan(Lq, Lk, H, hd, workspace is not None)
+    if SMS == 152 and plan:
+        units = -(-Lq // 256) * H
+        assert (got[0], got[3]) == (plan if workspace else (CONTIGUOUS if units <= SMS else WAVE, 0)), got
     q, k, v = (X.random_tensor(17, n + f"{r}x{d}", (r, d), std=s, bf16=True)
                for n, r, s in (("q", Lq, 1.5), ("k", Lk, 1.0), ("v", Lk, 1.0)))
     check(q, k, v, H, hd, workspace)
+
+
+# Waves whose two remaining units have fewer key tiles (142 at hd 64, 72 at hd
+# 128) than there are CTAs, some of which then get none of them: units 1216 and
+# 1217 = the last two query blocks of head 57, every row of them, and sampled rows
+# of other heads
+@pytest.mark.parametrize("Lk,hd", [(9060, 64), (4560, 128)])
+def test_attention_wave_remainder_of_few_tiles(Lk, hd):
+    Lq, H = 5300, 58
+    d = H * hd
+    if SMS == 152:
+        assert xb.debug_attention_plan(Lq, Lk, H, hd) == (WAVE, 152, 1, 2, 8)
+    q, k, v = (X.random_tensor(29, n + f"{r}x{d}", (r, d), std=s, bf16=True)
+               for n, r, s in (("q", Lq, 1.5), ("k", Lk, 1.0), ("v", Lk, 1.0)))
+    bf = lambda a: torch.from_numpy(a).to(DEV).to(torch.bfloat16)   # noqa: E731
+    o = torch.full((Lq + 64, d), 7.0, device=DEV, dtype=torch.bfloat16)
+    xb.op_attention("bf16", H, hd, bf(q), bf(k), bf(v), o[:Lq], workspace="auto")
+    got = o[:Lq].double().cpu().numpy()
+    for h, rows in ((57, np.arange(19 * 256, Lq)), (57, np.arange(0, 19 * 256, 97)), (0, np.arange(0, Lq, 61))):
+        cut = lambda a: a[:, h * hd:(h + 1) * hd].reshape(-1, 1, hd).astype(np.float64)   # noqa: E731
+        want = O.to_bf16(O.attention(cut(q[rows]), cut(k), cut(v)).reshape(len(rows), hd))
+        err = np.linalg.norm(got[rows, h * hd:(h + 1) * hd] - want, axis=1) / np.linalg.norm(want, axis=1)
+        assert np.sqrt(np.mean(err ** 2)) <= 5e-3 and err.max() <= 2e-2, (h, err.max())
+    assert bool((o[Lq:] == 7.0).all())
+    assert xb.op_device_error() == 0
 
 
 # A workspace that is not 16-byte aligned is not used (units whole): units that

@@ -258,14 +258,20 @@ def test_linear_full_size_sampled(M, N, K, epi):
         np.testing.assert_array_equal(host(rh), O.to_bf16(host(out) - xin))
 
 
-# Split-mode cases: more (head, 256-query) units than SMs, few key tiles, so
-# the CTA boundaries cut units at many different key tiles, including ragged
-# last tiles inside partial pieces; (8064, 100): one key tile, boundaries
-# never cut a unit.
-@pytest.mark.parametrize("Lq,Lk,H,hd", [(8064, 300, 8, 64), (8064, 700, 8, 64), (8064, 100, 8, 64),
-                                        (12960, 1000, 4, 128)])
-def test_attention_split_all_rows(Lq, Lk, H, hd):
+# More (head, 256-query) units than SMs, every row: cut contiguously (units just
+# above a multiple of 152 SMs), so that the CTA boundaries cut units at many
+# different key tiles, ragged last tiles inside partial pieces among them; and
+# few key tiles, where the units stay whole.
+@pytest.mark.parametrize("Lq,Lk,H,hd,cut", [(8064, 1000, 5, 64, True), (1300, 1500, 26, 64, True),
+                                            (8064, 700, 10, 64, True), (12960, 1800, 4, 128, True),
+                                            (8064, 300, 8, 64, False), (8064, 700, 8, 64, False),
+                                            (8064, 100, 8, 64, False), (12960, 1000, 4, 128, False)])
+def test_attention_split_all_rows(Lq, Lk, H, hd, cut):
     d = H * hd
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms == 152:
+        order, _, _, merged, _ = xb.debug_attention_plan(Lq, Lk, H, hd)
+        assert (order, merged) == ((0, 151) if cut else (1, 0))
     q = rt(f"Sq{Lq}{d}", (Lq, d))
     k = rt(f"Sk{Lk}{d}", (Lk, d))
     v = rt(f"Sv{Lk}{d}", (Lk, d))
