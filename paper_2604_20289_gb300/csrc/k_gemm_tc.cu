@@ -120,7 +120,8 @@ __device__ __forceinline__ void fma2(float &a, float &b, float x, float y, float
     a = t.x;
     b = t.y;
 }
-// gelu_tanh_approx of two values (the same operations, packed)
+// gelu_tanh of two values with the hardware tanh, packed: its relative error of
+// some 2^-11 is below the bf16 rounding of the output (2^-9)
 __device__ __forceinline__ void gelu_tanh_approx2(float &a, float &b) {
     const float k0 = 0.7978845608028654f;
     const float2 x = make_float2(a, b);

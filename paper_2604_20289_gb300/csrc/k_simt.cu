@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(SG_THREADS)
             v[2] += t.z;
             v[3] += t.w;
         }
-        epilogue_run<EPI, float, 4>(ep, m0 + r, n0 + c, v);
+        epilogue_run<EPI>(ep, m0 + r, n0 + c, v);
     }
 }
 
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(SG_THREADS)
     }
     if (n0 + c4 < ep.N) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) epilogue_run<EPI, float, 4>(ep, m0 + r4 + i, n0 + c4, acc[i]);
+        for (int i = 0; i < 4; ++i) epilogue_run<EPI>(ep, m0 + r4 + i, n0 + c4, acc[i]);
     }
 }
 

@@ -688,7 +688,6 @@ void run_pass(xc_ctx *ctx, const float *lat_dev, const float *action, float sigm
             ep.g_gw[q] = ctx->g_gw[q];
         }
         ep.frames = ctx->cfg.frames;
-        ep.frame0 = n * ctx->cfg.frames;
         ep.rope_axis = ctx->rope_axis;
         ep.rope_off = ctx->rope_off;
         ep.rope_cs = ctx->rope_cs;
@@ -1693,7 +1692,6 @@ xc_status xc_op_qkv_rope(int dtype, int n_cams, int frames, int gh, int gw, int 
     ep.d = d;
     ep.head_dim = head_dim;
     epi_single_grid(ep, frames, gh, gw);
-    ep.frame0 = chunk * frames;
     ep.rope_axis = axis;
     ep.rope_off = off;
     ep.rope_cs = cs;

@@ -165,19 +165,10 @@ __device__ __forceinline__ float gelu_tanh(float x) {
     const float k0 = 0.7978845608028654f;   // sqrt(2/pi)
     return 0.5f * x * (1.0f + tanhf(k0 * (x + 0.044715f * x * x * x)));
 }
-__device__ __forceinline__ float gelu_tanh_approx(float x) {
-    const float k0 = 0.7978845608028654f;
-    const float u = k0 * fmaf(0.044715f * x, x * x, x);
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-    const float hx = 0.5f * x;
-    return fmaf(hx, t, hx);
-}
 __device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
 
 // ------------------------------------------------------------ GEMM epilogue
-// Everything a fused GEMM epilogue may need.  One call processes the run of
-// 16 consecutive output columns [col, col + 16) of one row.
+// Everything a fused GEMM epilogue may need.
 struct EpiParams {
     int M, N;
     const float *bias;         // [N]
@@ -191,7 +182,7 @@ struct EpiParams {
     // RoPE geometry (QKV kind): view group g covers tokens [g_tok0[g],
     // g_tok0[g + 1]) with cameras g_cam0[g].. of g_npc[g] = frames * g_gh[g]
     // * g_gw[g] tokens each
-    int d, head_dim, frames, frame0;
+    int d, head_dim, frames;
     int n_groups;
     int g_tok0[XC_MAX_GROUPS], g_cam0[XC_MAX_GROUPS], g_npc[XC_MAX_GROUPS], g_gh[XC_MAX_GROUPS],
         g_gw[XC_MAX_GROUPS];
@@ -234,88 +225,43 @@ __device__ __forceinline__ int4 token_pos(const EpiParams &p, int row) {
 enum { EPI_BIAS = XC_EPI_BIAS, EPI_GELU = XC_EPI_GELU, EPI_RESID_GATE = XC_EPI_RESID_GATE,
        EPI_RESID_CACHE = XC_EPI_RESID_CACHE, EPI_QKV_ROPE = 16 };
 
-// Runs of W = 8 or 16 (float: also 4) consecutive elements (16-byte aligned).
-template <typename T, int W>
-__device__ __forceinline__ void loadW(const T *p, float (&v)[W]) {
-    if constexpr (W == 16) {
-        load16<T>(p, v);
-    } else if constexpr (sizeof(T) == 2) {
-        const uint4 u = *reinterpret_cast<const uint4 *>(p);
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[j]));
-            v[2 * j] = f.x;
-            v[2 * j + 1] = f.y;
-        }
-    } else if constexpr (W == 4) {
-        const float4 a = *reinterpret_cast<const float4 *>(p);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    } else {
-        const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    }
-}
-template <typename T, int W>
-__device__ __forceinline__ void storeW(T *p, const float (&v)[W]) {
-    if constexpr (W == 16) {
-        store16<T>(p, v);
-    } else if constexpr (sizeof(T) == 2) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-            w[j] = *reinterpret_cast<uint32_t *>(&h);
-        }
-        *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-    } else if constexpr (W == 4) {
-        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-        reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-        reinterpret_cast<float4 *>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
-    }
-}
-
-// Fused GEMM epilogue on one run of W consecutive output columns
-// [col, col + W) of one row (W = 4 (float), 8 or 16, col a multiple of W).
-template <int EPI, typename T, int W>
-__device__ __forceinline__ void epilogue_run(const EpiParams &p, int row, int col, float (&acc)[W]) {
+// Fused epilogue of the fp32 GEMMs on four consecutive output columns
+// [col, col + 4) of one row (col a multiple of 4, rows 16-byte aligned).
+template <int EPI>
+__device__ __forceinline__ void epilogue_run(const EpiParams &p, int row, int col, float (&acc)[4]) {
     if (row >= p.M) return;
-    {
-        float b[W];
-        loadW<float, W>(p.bias + col, b);
+    auto load = [](const void *base, size_t off, float (&v)[4]) {
+        const float4 t = *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(base) + off);
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    };
+    auto store = [&acc](void *base, size_t off) {
+        *reinterpret_cast<float4 *>(reinterpret_cast<float *>(base) + off) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    };
+    float b[4];
+    load(p.bias, col, b);
 #pragma unroll
-        for (int i = 0; i < W; ++i) acc[i] += b[i];
-    }
+    for (int i = 0; i < 4; ++i) acc[i] += b[i];
     const size_t off = (size_t)row * p.N + col;
     if constexpr (EPI == EPI_BIAS) {
-        storeW<T, W>(reinterpret_cast<T *>(p.out) + off, acc);
+        store(p.out, off);
     } else if constexpr (EPI == EPI_GELU) {
-        if constexpr (sizeof(T) == 2) {
-            // bf16 output: the hardware tanh (rel. error ~2^-11) is below the
-            // output rounding (2^-9)
 #pragma unroll
-            for (int i = 0; i < W; ++i) acc[i] = gelu_tanh_approx(acc[i]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < W; ++i) acc[i] = gelu_tanh(acc[i]);
-        }
-        storeW<T, W>(reinterpret_cast<T *>(p.out) + off, acc);
+        for (int i = 0; i < 4; ++i) acc[i] = gelu_tanh(acc[i]);
+        store(p.out, off);
     } else if constexpr (EPI == EPI_RESID_GATE || EPI == EPI_RESID_CACHE) {
-        float r[W], g[W];
-        loadW<T, W>(reinterpret_cast<const T *>(p.resid) + off, r);
-        loadW<float, W>(p.gate + col, g);
+        float r[4], g[4];
+        load(p.resid, off, r);
+        load(p.gate, col, g);
 #pragma unroll
-        for (int i = 0; i < W; ++i) acc[i] = r[i] + g[i] * acc[i];
-        storeW<T, W>(reinterpret_cast<T *>(p.out) + off, acc);
+        for (int i = 0; i < 4; ++i) acc[i] = r[i] + g[i] * acc[i];
+        store(p.out, off);
         if constexpr (EPI == EPI_RESID_CACHE) {
             if (p.rhat != nullptr) {
-                float xi[W];
-                loadW<T, W>(reinterpret_cast<const T *>(p.xin) + off, xi);
+                float xi[4];
+                load(p.xin, off, xi);
 #pragma unroll
-                for (int i = 0; i < W; ++i) acc[i] = round_to<T>(acc[i]) - xi[i];
-                storeW<T, W>(reinterpret_cast<T *>(p.rhat) + off, acc);
+                for (int i = 0; i < 4; ++i) acc[i] -= xi[i];
+                store(p.rhat, off);
             }
         }
     } else if constexpr (EPI == EPI_QKV_ROPE) {
@@ -327,7 +273,7 @@ __device__ __forceinline__ void epilogue_run(const EpiParams &p, int row, int co
             const int pos[4] = {tp.x, tp.y, tp.z, tp.w};      // frame: index within the chunk
             const int pair0 = (c % p.head_dim) >> 1;
 #pragma unroll
-            for (int j = 0; j < W / 2; ++j) {
+            for (int j = 0; j < 2; ++j) {
                 const int pr = pair0 + j;
                 const float2 t = p.rope_cs[p.rope_off[pr] + pos[p.rope_axis[pr]]];
                 const float x0 = acc[2 * j], x1 = acc[2 * j + 1];
@@ -335,8 +281,7 @@ __device__ __forceinline__ void epilogue_run(const EpiParams &p, int row, int co
                 acc[2 * j + 1] = x0 * t.y + x1 * t.x;
             }
         }
-        T *dst = reinterpret_cast<T *>(part == 0 ? p.out : (part == 1 ? p.out_k : p.out_v));
-        storeW<T, W>(dst + (size_t)row * d + c, acc);
+        store(part == 0 ? p.out : (part == 1 ? p.out_k : p.out_v), (size_t)row * d + c);
     }
 }
 }  // namespace xc

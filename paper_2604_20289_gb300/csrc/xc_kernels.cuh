@@ -95,12 +95,11 @@ struct WeightMaps {
 // Tiling of gemm_tc_bn: 64, 128 (single CTAs), 256 (CTA pairs), GEMM_WIDE
 // (single CTAs, 256 columns).
 constexpr int GEMM_WIDE = 257;
-// The maps that tiling bn uses (0: all).
+// The maps that tiling bn uses.
 inline bool make_weight_maps(WeightMaps *m, int bn, const void *base, uint64_t N, uint64_t K) {
-    const bool all = bn == 0;
-    return (!(all || bn == 128 || bn == 256) || make_tmap_bf16(&m->box128, base, N, K, 128)) &&
-           (!(all || bn == 64 || bn == 256) || make_tmap_bf16(&m->box64, base, N, K, 64)) &&
-           (!(all || bn == GEMM_WIDE) || make_tmap_bf16(&m->box256, base, N, K, 256));
+    return (!(bn == 128 || bn == 256) || make_tmap_bf16(&m->box128, base, N, K, 128)) &&
+           (!(bn == 64 || bn == 256) || make_tmap_bf16(&m->box64, base, N, K, 64)) &&
+           (bn != GEMM_WIDE || make_tmap_bf16(&m->box256, base, N, K, 256));
 }
 int gemm_tc_bn(int epi, int M, int N, int K);
 void gemm_tc_tiles(int bn, int M, int N, int *full, int *half);    // of that tiling
