@@ -1515,15 +1515,18 @@ xc_status xc_chunk_step(xc_ctx *ctx, const float *latent, const float *action, f
 // Error word of the operator entry points on the current device, made by the
 // first call on it.
 static int *op_err_word() {
+    static std::atomic<int *> words[PerDevice::MAX];
     static std::mutex mu;
-    static std::map<int, int *> words;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= PerDevice::MAX) return nullptr;
+    int *p = words[dev].load(std::memory_order_acquire);
+    if (p != nullptr) return p;
     std::lock_guard<std::mutex> lk(mu);
-    int *&p = words[dev];
+    p = words[dev].load(std::memory_order_relaxed);
     if (p == nullptr) {
-        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) return p = nullptr;
+        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess) return nullptr;
         cudaMemset(p, 0, sizeof(int));
+        words[dev].store(p, std::memory_order_release);
     }
     return p;
 }
