@@ -49,7 +49,7 @@ CONTIGUOUS, WAVE, CLUSTER = 0, 1, 2
 ORDERS = [
     (840, 2520, 4, 64, (CLUSTER, 0)),            # 16 units in clusters of 8
     (130, 5000, 1, 128, (CLUSTER, 0)),           # one unit
-    (1400, 1000, 7, 64, (CLUSTER, 0)),           # 42 units in clusters of 3
+    (700, 1000, 13, 64, (CLUSTER, 0)),           # 39 units in clusters of 3
     (600, 1450, 2, 128, (CLUSTER, 0)),           # 6 in clusters of 6
     (840, 2520, 6, 128, None),                   # 24 in clusters of 6 where so many fit, else split 6 ways
     (300, 9000, 2, 128, (WAVE, 4)),              # 4 units split 15 ways
